@@ -210,10 +210,12 @@ bsm_status bsm_get_launch_count(int64_t *count);
 /* Numeric variant per precision and output block shape (m rows, n columns),
  * for tiny blocks (m*n <= 16, 5 x 5, and on the FP64 and Ozaki paths 6 x 6;
  * other shapes always use variant 0):
- * 0 = one warp per output block (FP64: lanes over its elements; split and
- * Ozaki paths: tensor-core MMA on packed fragments), 1 = one lane per output
- * block on CUDA cores (split paths: the same split pieces multiplied with FP32
- * FMA, exact piece products; Ozaki path: plain FP64 FMA).  -1 restores the
+ * 0 = one warp per output block (FP64_DMMA and FP32 data: lanes over its
+ * elements; split and Ozaki paths: tensor-core MMA on packed fragments), 1 =
+ * one lane per output block on CUDA cores (split paths: the same split pieces
+ * multiplied with FP32 FMA, exact piece products; Ozaki path: plain FP64 FMA).
+ * BSM_P_FP64 on FP64 data chooses the lanes of a block itself, whatever is set
+ * here (the results are the same bits for any choice).  -1 restores the
  * library default (1 for m*n <= 16, 0 for 5 x 5 and 6 x 6);
  * bsm_get_variant returns the variant in effect.
  * Process-wide; the autotuner (paper_1708_03604_gb300/autotune.py) sets it
@@ -250,7 +252,7 @@ bsm_status bsm_get_variant(int32_t prec, int32_t m, int32_t n, int32_t *variant)
  *                        fewer registers), FP64_DMMA 1..3 (default 3)
  *   BSM_TUNE_FP64_BUILD  BSM_P_FP64 only: FP64 FMA kernel build, 0 chosen by
  *                        the largest output block (default), 1 narrow (up to
- *                        9 elements per lane per pass), 2 wide (up to 24);
+ *                        13 elements per lane per pass), 2 wide (up to 24);
  *                        output blocks of at most 16 elements always run the
  *                        small build
  *   BSM_TUNE_SCHED_TILE  order of the output blocks inside a block-shape

@@ -1635,6 +1635,8 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
     // split paths: blocks of one tile row in their own kernel instance, unless
     // the tuning fixes the pass rows; Ozaki path: blocks of one tile column
     const bool want_groups = rprec == BSM_P_OZAKI || tune_of(rprec)[BSM_TUNE_PASS_MT] <= 0;
+    // the FP64 kernel groups small blocks by itself: no variant marks in its order
+    const int order_prec = kprec == BSM_P_FP64 && A->dtype == BSM_FP64 ? -1 : rprec;
     auto numeric_pass = [&](int64_t cb0, int64_t nitems, int64_t nprod_pass, bool whole) -> bsm_status {
         NumericArgs na{};
         na.n_items = nitems;
@@ -1674,11 +1676,11 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
             rows_view.nbr = nbr;
             rows_view.row_ptr = crow_ptr;
             if ((sst = shape_order(sc, nitems, c_rc + cb0, A->h_row_bs, B->h_col_bs, &order, &rows_view, A->row_rank,
-                                   rprec, &uses_cores, &n_marked, c_col + cb0, tile > 0 ? B->col_rank : nullptr, nbc,
+                                   order_prec, &uses_cores, &n_marked, c_col + cb0, tile > 0 ? B->col_rank : nullptr, nbc,
                                    tile > 0 ? tile : 0, want_groups ? &groups : nullptr)))
                 return sst;
         } else {  // a row panel: block-shape classes and variants only
-            if ((sst = shape_order(sc, nitems, c_rc + cb0, A->h_row_bs, B->h_col_bs, &order, nullptr, nullptr, rprec,
+            if ((sst = shape_order(sc, nitems, c_rc + cb0, A->h_row_bs, B->h_col_bs, &order, nullptr, nullptr, order_prec,
                                    &uses_cores, &n_marked, nullptr, nullptr, 0, 0, want_groups ? &groups : nullptr)))
                 return sst;
         }
@@ -1941,7 +1943,7 @@ bsm_status bsm_multiply_backward(double alpha, bsm_t C, const void *dC_data, bsm
         int64_t *n_marked = nullptr;
         bool uses_cores = false;
         if ((st = shape_order(sc, OUT->nnzb, OUT->blk_rc, OUT->h_row_bs, OUT->h_col_bs, &item_order, nullptr, nullptr,
-                              opts.prec, &uses_cores, &n_marked)))
+                              kprec == BSM_P_FP64 && C->dtype == BSM_FP64 ? -1 : opts.prec, &uses_cores, &n_marked)))
             return st;
         na.n_lane_items = n_marked;
         if (needs_plain(kprec) && uses_cores && nprod > 0) {

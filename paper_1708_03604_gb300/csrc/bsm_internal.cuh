@@ -260,6 +260,7 @@ struct NumericArgs {
     double alpha, beta;
     const void *old_data;       // beta != 0: old values at old_off[q] (or -1)
     const int64_t *old_off;
+    int32_t unit_alpha, has_old;  // alpha == 1; beta != 0 with old blocks (set by launch_numeric)
     int32_t dtype;
     int32_t prec;
     int32_t flush_every;
@@ -305,6 +306,12 @@ struct NumericLaunch {
     int32_t cta_threads, grid, pass_mt, pass_nt;
 };
 cudaError_t launch_numeric(const NumericArgs &a, cudaStream_t s, NumericLaunch *info = nullptr);
+// Builds of the CUDA-core kernels by the largest output block (elements a lane holds)
+constexpr int kCcSmall = 0, kCcNarrow = 1, kCcWide = 2;
+// FP64 data on the CUDA cores (k_group.cu); *grid: CTAs launched
+cudaError_t launch_numeric_group(const NumericArgs &a, int build, cudaStream_t s, int *grid);
+uint32_t group_debug_bits(cudaStream_t s);
+int num_sms();
 // out[g] = number of keys below thr[g] in the ascending keys[0..n) (g < 2)
 cudaError_t launch_group_bounds(const uint32_t *keys, int64_t n, uint32_t thr0, uint32_t thr1, int64_t *out,
                                 cudaStream_t s);
