@@ -698,7 +698,6 @@ struct PanelOut {
     int64_t nnzbC;
     const int64_t *c_row_ptr;
     const int32_t *c_col;
-    const int64_t *c_off;
     double *c_data;
     const int64_t *old_off;  // null unless beta != 0
     const void *old_data;
@@ -781,8 +780,8 @@ bsm_status run_panel(Scratch &sc, bsm_mat *A, bsm_mat *B, int32_t s, const Panel
     if (e == cudaSuccess) e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), g_stream);
     if ((st = cuda_check(e, "panel operands"))) return st;
     pa.a_pack = apk; pa.b_pack = bpk; pa.zeros = zeros;
-    pa.c_data = o.c_data; pa.c_blk_off = o.c_off;
-    pa.alpha = o.alpha; pa.beta = o.beta;
+    pa.c_data = o.c_data;
+    pa.alpha = o.alpha; pa.beta = o.beta; pa.unit_alpha = o.alpha == 1.0;
     pa.old_data = o.old_data; pa.old_off = o.old_off;
     pa.status = o.status;
     pa.work_counter = counter;
@@ -1608,7 +1607,7 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
     int64_t *n_marked = nullptr, *groups = nullptr;
     bool uses_cores = false;
     if (use_panel) {
-        PanelOut po{nnzbC, crow_ptr, c_col, c_off, static_cast<double *>(c_data), old_off,
+        PanelOut po{nnzbC, crow_ptr, c_col, static_cast<double *>(c_data), old_off,
                     use_old ? C->data : nullptr, alpha, use_old ? beta : 0.0, C->status};
         if ((st = run_panel(sc, A, B, panel_s, po, ev, opts.prec))) return st;
         int32_t hs = 0;

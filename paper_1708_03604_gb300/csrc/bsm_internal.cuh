@@ -423,8 +423,9 @@ struct PanelArgs {
     // block indices (A's 5 row slots, then B's 5 column slots; -1: absent)
     const int64_t *step_ptr;
     int32_t *steps;
-    double *c_data; const int64_t *c_blk_off;
+    double *c_data;                       // block q at q * s * s
     double alpha, beta;
+    int32_t unit_alpha;                   // alpha == 1
     const void *old_data; const int64_t *old_off;  // beta != 0: old values (or null)
     int32_t *status;                      // set to BSM_ERR_TIMEOUT when a wait gives up
     unsigned long long *work_counter;     // zeroed by the caller

@@ -24,24 +24,34 @@
 // The k-steps of every tile (a merge of its five A rows' and five B columns'
 // sorted block-index lists) are written beforehand by k_panel_steps, one warp
 // per tile, as records of 10 block indices.  Roles in one persistent CTA per
-// SM of the numeric kernel (12 warps):
+// SM of the numeric kernel (25 warps):
 //   warp 0      tickets: takes tiles from an atomic ticket and hands each,
-//               with its range of k-step records, to the copy warps through a
-//               shared ring;
+//               with its range of k-step records, to the copy and MMA warps
+//               through a shared ring;
 //   warps 1, 2  copy: stage the 10 blocks of every k-step (warp 1 A's, warp 2
-//               B's; the block indices of 32 k-steps per coalesced load), one
-//               bulk copy of 4608 bytes per block pre-packed in the tensor
-//               core's shared-memory layout (absent blocks from a zero block),
-//               completion counted in bytes on the stage's "full" barrier
-//               (4-stage ring);
-//   warp 3      allocates tensor memory; one lane issues the MMAs of a k-step
-//               into accumulator buffer b and commits them to the stage's
-//               "empty" barrier and, every third k-step, to the buffer's
-//               "full" barrier;
-//   warps 4..11 drain: each owns one 32-lane quarter of tensor memory (32 rows
-//               of the tile) and one half of its columns, reads the buffer
-//               into registers, frees it, adds it into the compensated pair,
-//               and on a tile's last k-step writes C.
+//               B's; the block indices two k-steps ahead), one
+//               bulk copy of 4608 bytes per present block, pre-packed in the
+//               tensor core's shared-memory layout, completion counted in bytes
+//               on the stage's "full" barrier (4-stage ring); the slots of
+//               absent blocks take a zero block unless they hold one;
+//   warps 3, 24 MMA: groups of k-steps in turn (warp 3 also allocates tensor
+//               memory); one lane issues the MMAs of a k-step into the group's
+//               accumulator buffer (of four, all of tensor memory) and commits
+//               them to the stage's "empty" barrier and, after a group (three
+//               k-steps by default), to the buffer's "full" barrier;
+//   warps 4..23 drain: each owns one 32-lane quarter of tensor memory (32 rows
+//               of the tile) and one column slot, reads the buffer into
+//               registers, frees it, adds it into the compensated pair, and on
+//               a tile's last k-step writes C.
+// What bounds it: a k-step's 9 MMAs need about 600 cycles of the tensor core; the
+// chain of waits, issue and commits of one MMA warp took 1,000 and the drain
+// competed with it.  On 2,000 banded block rows (2.0e7 products of 23 x 23, 3.1e6
+// k-steps) the kernel went from 16.6 ms to 10.9: 20 drain warps of one column
+// slot in place of 8 of 64 columns (80 registers instead of 168, five warps a
+// scheduler: 15.8 -> 12.4), two MMA warps (-> 12.0), paired FP32 instructions
+// in the drain (-> 10.9), four accumulator buffers, integer conversion.  The
+// copies are not the limit: without them it takes the same time.
+//
 // Every wait is bounded (2 s by default; the main-loop waits take
 // PanelArgs::wait_ns, which tests shorten to make a wait run out); a wait that
 // runs out sets the output's status word to BSM_ERR_TIMEOUT, every role then
@@ -73,11 +83,12 @@ constexpr int kBlk = 3 * kGroupStride;    // bytes of one packed block (hi and l
 constexpr int kOperand = 16 * kGroupStride;  // one operand of a stage, 128 rows: 24576
 constexpr int kStageBytes = 2 * kOperand;    // A, then B
 constexpr int kStages = 4;
-constexpr int kRing = 8;                  // tiles handed from the ticket warp to the copy warps
+constexpr int kRing = 8;                  // tiles handed from the ticket warp to the copy and MMA warps
 constexpr int kPre = 4;                   // list entries the merge loads ahead
+constexpr int kAcc = 4;                   // accumulator buffers (128 tensor-memory columns each)
 constexpr int kPair = 3;                  // default k-steps summed in one accumulator buffer before a drain
-constexpr int kCopyWarps = 2, kMmaWarp = 3, kDrainWarps = 8;
-constexpr int kThreads = 32 * (2 + kCopyWarps + kDrainWarps);
+constexpr int kCopyWarps = 2, kMmaWarp = 3, kDrainWarps = 4 * kCB, kMmaWarp2 = kMmaWarp + kDrainWarps + 1;
+constexpr int kThreads = 32 * (kMmaWarp2 + 1);
 constexpr unsigned long long kWaitNs = 2000000000ull;  // a wait gives up after 2 s
 // instruction descriptor: D F32, A and B TF32, both K-major, N = 128, M = 128
 constexpr uint32_t kIdesc = (1u << 4) | (2u << 7) | (2u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
@@ -85,14 +96,19 @@ constexpr int kFirst = 1, kLast = 2, kDone = 4;
 
 __device__ __forceinline__ uint32_t saddr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// one lane of a converged warp, the same one every time
+__device__ __forceinline__ bool elect_one() {
+    uint32_t is;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xFFFFFFFF;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(is));
+    return is != 0;
+}
+
 // shared-memory matrix descriptor, no swizzle: 8-row x 16-byte core matrices,
-// `lbo` bytes between core matrices along K, `sbo` bytes along M / N
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = (uint64_t)((addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-    d |= (uint64_t)1 << 46;  // descriptor version of the fifth-generation tensor cores
-    return d;
+// `low` the address and the bytes between core matrices along K, both in
+// 16-byte units; kGroupStride bytes between them along M / N
+__device__ __forceinline__ uint64_t sdesc(uint32_t low) {
+    constexpr uint32_t high = (kGroupStride >> 4) | (1u << 14);  // bit 46: fifth-generation tensor cores
+    return (uint64_t)high << 32 | low;
 }
 
 __device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t a, uint64_t b, int accumulate) {
@@ -133,11 +149,19 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, const 
                                           unsigned long long limit_ns = kWaitNs) {
     // each try_wait suspends the thread (no issue slots taken) until the
     // phase completes or the hinted time (20 us, less under a shorter limit)
-    // passes
+    // passes; the timer is read only after one that did not complete
     const uint32_t hint = limit_ns < 20000ull ? (uint32_t)limit_ns : 20000u;
-    const unsigned long long t0 = global_ns();
+    unsigned long long t0 = 0;
+    uint32_t ok;
+    if (limit_ns == 0) {
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok)
+            : "r"(mbar), "r"(parity)
+            : "memory");
+        return ok != 0;
+    }
     for (;;) {
-        uint32_t ok;
         asm volatile(
             "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
             : "=r"(ok)
@@ -145,34 +169,52 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, const 
             : "memory");
         if (ok) return true;
         if (*(volatile const int32_t *)abort) return false;
-        if (global_ns() - t0 > limit_ns) return false;
+        const unsigned long long now = global_ns();
+        if (t0 && now - t0 > limit_ns) return false;
+        if (!t0) t0 = now;
     }
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t *r) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // compensated add of b into (hi, lo) (the update of the mma.sync TF32x3
 // path) with the compensation lo held as BF16: lo is below half an ulp of hi,
-// so rounding it to 8 bits costs at most 2^-9 of it, 2^-33 of hi, per add
-__device__ __forceinline__ void kahan_b2(float &hi0, float &hi1, __nv_bfloat162 &lo, float b0, float b1) {
+// so rounding it to 8 bits costs at most 2^-9 of it, 2^-33 of hi, per add.
+// Two elements at a time in paired FP32 instructions: the drain warps share
+// their schedulers with the MMA warps, whose issue they slow down.
+__device__ __forceinline__ uint64_t pack2(float x, float y) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t x, uint64_t y) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+    return r;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t x, uint64_t y) {
+    uint64_t r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+    return r;
+}
+__device__ __forceinline__ void kahan_b2(uint64_t &hi, __nv_bfloat162 &lo, uint64_t b) {
     const float2 l = __bfloat1622float2(lo);
-    const float y0 = __fadd_rn(b0, l.x), y1 = __fadd_rn(b1, l.y);
-    const float t0 = __fadd_rn(hi0, y0), t1 = __fadd_rn(hi1, y1);
-    lo = __floats2bfloat162_rn(__fsub_rn(y0, __fsub_rn(t0, hi0)), __fsub_rn(y1, __fsub_rn(t1, hi1)));
-    hi0 = t0;
-    hi1 = t1;
+    const uint64_t y = add2(b, pack2(l.x, l.y)), t = add2(hi, y);
+    const float2 d = unpack2(sub2(y, sub2(t, hi)));
+    lo = __floats2bfloat162_rn(d.x, d.y);
+    hi = t;
 }
 
 __device__ __forceinline__ uint32_t to_tf32(float x) {
@@ -317,12 +359,11 @@ struct TileRec {
 
 struct SmemCtl {
     uint64_t full[kStages], empty[kStages];
-    uint64_t accf[2], acce[2];
+    uint64_t accf[kAcc], acce[kAcc];
     uint64_t rec_full[kRing], rec_empty[kRing];
-    uint64_t fin;
+    uint64_t fin[2];
     TileRec rec[kRing];
-    int32_t smeta_t[kStages], smeta_f[kStages];
-    int32_t ameta_t[2], ameta_f[2];
+    int32_t ameta_t[kAcc], ameta_f[kAcc];
     uint32_t tmem;
     int32_t abort;
 };
@@ -529,18 +570,49 @@ __global__ void __launch_bounds__(128) k_panel_steps_bm(PanelArgs a, int fill, i
     }
 }
 
-// Drain warp of tensor-memory lanes 32 quarter .. +31 (tile rows) and columns
-// 64 HALF .. +63 of both accumulator buffers: its threads keep the compensated
-// pair of their 64 elements in registers (sum FP32, compensation BF16), add
-// every buffer into it, and on a tile's last k-step write the tile's C blocks.
-template <int HALF>
-__device__ __forceinline__ void drain(const PanelArgs &a, SmemCtl &ctl, uint32_t tmem, int quarter, int lane,
+// hi + lo in FP64, lo the BF16 compensation (at most half an ulp of hi) in the
+// low 16 bits of `lo`: the sum of the two significands as integers, hi's 24
+// bits at 2^29 of a 53-bit one.  The sum is exact there whenever lo's lowest
+// bit is not below the 53rd (else, and for zero, subnormal and non-finite hi,
+// an FP64 addition), so it is what the FP64 addition gives, without the FP64
+// pipe: two conversions and an addition per element there took 37,000 cycles a
+// tile, in which the tensor core waited for the drain.
+__device__ __forceinline__ double pair_value(float hi, uint32_t lo) {
+    const uint32_t h = __float_as_uint(hi);
+    const uint32_t eh = (h >> 23) & 0xffu, el = (lo >> 7) & 0xffu;
+    const bool none = (lo & 0x7fffu) == 0u;
+    const int s = (int)el - (int)eh + 45;  // place of lo's lowest bit
+    if (eh - 1u >= 254u || (!none && (el == 0u || s < 0 || s > 21)))
+        return (double)hi + (double)__uint_as_float(lo << 16);
+    const uint32_t part = none ? 0u : ((lo & 0x7fu) | 0x80u) << s;  // below 2^29
+    const unsigned long long m = (unsigned long long)((h & 0x7fffffu) | 0x800000u) << 29;
+    unsigned long long sum = (h ^ (lo << 16)) >> 31 ? m - part : m + part;
+    uint32_t e = eh + (1023 - 127);
+    if (!(sum >> 52)) {
+        sum <<= 1;
+        --e;
+    }
+    return __longlong_as_double((long long)((unsigned long long)(h & 0x80000000u) << 32 | (unsigned long long)e << 52 |
+                                            (sum & 0xfffffffffffffull)));
+}
+
+// Drain warp of tensor-memory lanes 32 quarter .. +31 (tile rows) and the 24
+// columns of column slot `c` of every accumulator buffer: its threads keep the
+// compensated pair of their 24 elements in registers (sum FP32, compensation
+// BF16), add every buffer into it, and on a tile's last k-step write their
+// rows of the tile's C blocks in that slot.
+__device__ __forceinline__ void drain(const PanelArgs &a, SmemCtl &ctl, uint32_t tmem, int quarter, int c, int lane,
                                       bool dead) {
     const int row = quarter * 32 + lane;
     const int si = row / kSlot, ri = row - si * kSlot;
-    const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16) + HALF * 64;
-    float sh[64];
-    __nv_bfloat162 sl[32];  // compensation of elements 2i, 2i + 1
+    const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16) + c * kSlot;
+    uint64_t sh[kSlot / 2];        // sums of elements 2i, 2i + 1
+    __nv_bfloat162 sl[kSlot / 2];  // and their compensation
+#pragma unroll
+    for (int e = 0; e < kSlot / 2; ++e) {
+        sh[e] = 0;
+        sl[e] = __floats2bfloat162_rn(0.f, 0.f);
+    }
     uint32_t buf = 0, bph = 0;
     bool ok = !dead;
     while (ok) {
@@ -551,53 +623,42 @@ __device__ __forceinline__ void drain(const PanelArgs &a, SmemCtl &ctl, uint32_t
         tc_fence_after();
         const int32_t t = ctl.ameta_t[buf], flags = ctl.ameta_f[buf];
         if (flags & kDone) break;
-        const bool first = flags & kFirst, last = flags & kLast;
+        // the lane's C block, under way while the buffer is added
+        int32_t q = -1;
+        if ((flags & kLast) && si < kRB && ri < a.s) q = a.cblk[(int64_t)t * (kRB * kCB) + si * kCB + c];
+        uint32_t v[kSlot];
 #pragma unroll
-        for (int ch = 0; ch < 2; ++ch) {
-            uint32_t v[32];
-            tmem_ld32(lane_base + buf * 128 + ch * 32, v);
-            tmem_wait_ld();
-            if (ch == 1) {  // the buffer is free as soon as it is in registers
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(saddr(&ctl.acce[buf]));
-            }
+        for (int ch = 0; ch < kSlot; ch += 8) tmem_ld8(base + buf * 128 + ch, v + ch);
+        tmem_wait_ld();
+        tc_fence_before();  // the buffer is free as soon as it is in registers
+        __syncwarp();
+        if (lane == 0) mbar_arrive(saddr(&ctl.acce[buf]));
 #pragma unroll
-            for (int e = 0; e < 32; e += 2) {
-                if (first) {  // the compensated add of v into (0, 0)
-                    sh[ch * 32 + e] = __uint_as_float(v[e]);
-                    sh[ch * 32 + e + 1] = __uint_as_float(v[e + 1]);
-                    sl[(ch * 32 + e) / 2] = __floats2bfloat162_rn(0.f, 0.f);
-                } else {
-                    kahan_b2(sh[ch * 32 + e], sh[ch * 32 + e + 1], sl[(ch * 32 + e) / 2], __uint_as_float(v[e]),
-                             __uint_as_float(v[e + 1]));
-                }
+        for (int e = 0; e < kSlot / 2; ++e) {
+            const uint64_t b = pack2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
+            if (flags & kFirst) {  // the compensated add of b into (0, 0)
+                sh[e] = b;
+                sl[e] = __floats2bfloat162_rn(0.f, 0.f);
+            } else {
+                kahan_b2(sh[e], sl[e], b);
             }
         }
-        buf ^= 1u;
+        buf = (buf + 1) % kAcc;
         if (buf == 0) bph ^= 1u;
-        if (last && si < kRB && ri < a.s) {
-            const double *old = static_cast<const double *>(a.old_data);
-            const int32_t *cb = a.cblk + (int64_t)t * (kRB * kCB) + si * kCB;
-            // the column slots this half of the tile touches
-            constexpr int c0 = (HALF * 64) / kSlot, c1 = (HALF * 64 + 63) / kSlot;
+        if (q >= 0) {
+            // C's blocks have one size and lie one after the other
+            double *out = a.c_data + (int64_t)q * (a.s * a.s) + ri * a.s;
+            const int64_t oo = a.old_data && a.old_off ? a.old_off[q] : -1;
+            const double *old = static_cast<const double *>(a.old_data) + oo + (int64_t)ri * a.s;
 #pragma unroll
-            for (int c = c0; c <= c1 && c < kCB; ++c) {
-                const int32_t q = cb[c];
-                if (q < 0) continue;
-                const int64_t o = a.c_blk_off[q] + (int64_t)ri * a.s;
-                const int64_t oo = (old && a.old_off) ? a.old_off[q] : -1;
-#pragma unroll
-                for (int e = 0; e < 64; ++e) {
-                    const int col = HALF * 64 + e;
-                    if (col / kSlot != c) continue;
-                    const int cj = col - c * kSlot;
-                    if (cj >= a.s) continue;
-                    const float2 lo = __bfloat1622float2(sl[e / 2]);
-                    double val = a.alpha * ((double)sh[e] + (double)((e & 1) ? lo.y : lo.x));
-                    if (oo >= 0) val = fma(a.beta, old[oo + (int64_t)ri * a.s + cj], val);
-                    a.c_data[o + cj] = val;
-                }
+            for (int e = 0; e < kSlot; ++e) {
+                if (e >= a.s) break;
+                const uint32_t lo = *reinterpret_cast<const uint32_t *>(&sl[e / 2]);
+                const float2 hi = unpack2(sh[e / 2]);
+                double val = (e & 1) ? pair_value(hi.y, lo >> 16) : pair_value(hi.x, lo & 0xffffu);
+                if (!a.unit_alpha) val *= a.alpha;
+                if (oo >= 0) val = fma(a.beta, old[e], val);
+                out[e] = val;
             }
         }
     }
@@ -618,17 +679,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_panel_tf32x3(PanelArgs a) {
     if (threadIdx.x == 0) {
         for (int st = 0; st < kStages; ++st) {
             mbar_init(saddr(&ctl.full[st]), kCopyWarps);
-            mbar_init(saddr(&ctl.empty[st]), 1);
+            mbar_init(saddr(&ctl.empty[st]), 2);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < kAcc; ++b) {
             mbar_init(saddr(&ctl.accf[b]), 2);
             mbar_init(saddr(&ctl.acce[b]), kDrainWarps);
         }
         for (int r = 0; r < kRing; ++r) {
             mbar_init(saddr(&ctl.rec_full[r]), 1);
-            mbar_init(saddr(&ctl.rec_empty[r]), kCopyWarps);
+            mbar_init(saddr(&ctl.rec_empty[r]), kCopyWarps + 2);
         }
-        mbar_init(saddr(&ctl.fin), 1);
+        for (int w = 0; w < 2; ++w) mbar_init(saddr(&ctl.fin[w]), 1);
         ctl.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -648,7 +709,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_panel_tf32x3(PanelArgs a) {
     if (warp == 0) {
         // ------------------------------------------------------------ tiles
         // hands the tiles of the atomic ticket, with their k-step ranges, to
-        // the copy warps through the ring
+        // the copy and MMA warps through the ring
         uint32_t rs = 0, rph = 0;
         bool ok = !dead;
         for (;;) {
@@ -681,14 +742,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_panel_tf32x3(PanelArgs a) {
     } else if (warp <= kCopyWarps) {
         // ------------------------------------------------------------ copy
         // warp 1 stages A's 5 blocks of every k-step, warp 2 B's: one bulk
-        // copy of 4608 bytes per block (absent blocks from a zero block),
-        // completion counted in bytes on the stage's "full" barrier.  The
-        // block indices of 32 k-steps come in with one load per lane.
+        // copy of 4608 bytes per present block, completion counted in bytes on
+        // the stage's "full" barrier; the slots of absent blocks (about half of
+        // them on a half-filled band) take a copy of a zero block, and only when
+        // the stage's last step left a block there.  The block indices
+        // come in two k-steps ahead.
         const int cw = warp - 1;
         const bool is_a = cw == 0;
         const uint8_t *pk = is_a ? a.a_pack : a.b_pack;
         uint32_t st = 0, ph = 0, rs = 0, rph = 0;
         int64_t issued = 0;
+        uint32_t zeroed = 0;  // bit 5 st + q: slot q of stage st holds zeros
         bool ok = !dead;
         while (ok) {
             if (!__all_sync(0xffffffffu, mbar_wait(saddr(&ctl.rec_full[rs]), rph, &ctl.abort, a.wait_ns))) {
@@ -703,56 +767,35 @@ __global__ void __launch_bounds__(kThreads, 1) k_panel_tf32x3(PanelArgs a) {
                 rs = 0;
                 rph ^= 1u;
             }
-            if (r.tile < 0) {  // the end marker for the MMA lane
+            if (r.tile < 0) break;
+            // lanes 0 .. 4 hold the block index of their slot, two steps ahead
+            const int32_t *idx = a.steps + (is_a ? 0 : kRB) + lane;
+            auto index_at = [&](int64_t s) { return lane < kRB && s < r.s1 ? __ldg(idx + s * (kRB + kCB)) : -1; };
+            int32_t blk = -1, blk1 = index_at(r.s0), blk2 = index_at(r.s0 + 1);
+            for (int64_t s = r.s0; s < r.s1; ++s) {
+                blk = blk1;
+                blk1 = blk2;
+                blk2 = index_at(s + 2);
+                // absent blocks: zeros where the slot does not hold them yet
+                constexpr uint32_t kAll = (1u << kRB) - 1u;
+                const uint32_t present = __ballot_sync(0xffffffffu, blk >= 0);
+                const uint32_t copies = present | (~(zeroed >> (kRB * st)) & kAll);
+                zeroed = (zeroed & ~(kAll << (kRB * st))) | ((~present & kAll) << (kRB * st));
                 if (!__all_sync(0xffffffffu, mbar_wait(saddr(&ctl.empty[st]), ph ^ 1u, &ctl.abort, a.wait_ns))) {
                     if (lane == 0) fail(ctl, a.status);
                     ok = false;
                     break;
                 }
-                if (lane == 0) {
-                    if (is_a) ctl.smeta_f[st] = kDone;
-                    mbar_arrive(saddr(&ctl.full[st]));
-                }
-                break;
-            }
-            for (int64_t base = r.s0; base < r.s1 && ok; base += 32) {
-                // lane l: the 5 block indices of this warp's operand for k-step base + l
-                int32_t f[kRB];
-                const int64_t sl = base + lane;
-#pragma unroll
-                for (int q = 0; q < kRB; ++q) f[q] = sl < r.s1 ? a.steps[sl * (kRB + kCB) + (is_a ? 0 : kRB) + q] : -1;
-                const int n = (int)(r.s1 - base < 32 ? r.s1 - base : 32);
-                for (int j = 0; j < n; ++j) {
-                    int32_t blk = -1;
-#pragma unroll
-                    for (int q = 0; q < kRB; ++q) {
-                        const int32_t x = __shfl_sync(0xffffffffu, f[q], j);
-                        if (lane == q) blk = x;
-                    }
-                    if (!__all_sync(0xffffffffu, mbar_wait(saddr(&ctl.empty[st]), ph ^ 1u, &ctl.abort, a.wait_ns))) {
-                        if (lane == 0) fail(ctl, a.status);
-                        ok = false;
-                        break;
-                    }
-                    if (lane == 0) {
-                        if (is_a) {
-                            const int64_t sidx = base + j;
-                            ctl.smeta_t[st] = r.tile;
-                            ctl.smeta_f[st] = (sidx == r.s0 ? kFirst : 0) | (sidx + 1 == r.s1 ? kLast : 0);
-                        }
-                        mbar_arrive_tx(saddr(&ctl.full[st]), kRB * kBlk);
-                    }
-                    __syncwarp();
-                    if (lane < kRB) {
-                        const void *src = blk >= 0 ? (const void *)(pk + (int64_t)blk * kBlk) : (const void *)a.zeros;
-                        bulk_copy(saddr(stages + st * kStageBytes + (is_a ? 0 : kOperand) + lane * kBlk), src, kBlk,
-                                  saddr(&ctl.full[st]));
-                    }
-                    ++issued;
-                    if (++st == kStages) {
-                        st = 0;
-                        ph ^= 1u;
-                    }
+                const uint32_t full = saddr(&ctl.full[st]);
+                if (lane == 0) mbar_arrive_tx(full, (uint32_t)__popc(copies) * kBlk);
+                __syncwarp();
+                if ((copies >> lane) & 1u)  // lanes 0 .. 4
+                    bulk_copy(saddr(stages) + st * kStageBytes + (is_a ? 0 : kOperand) + lane * kBlk,
+                              blk >= 0 ? pk + (int64_t)blk * kBlk : a.zeros, kBlk, full);
+                ++issued;
+                if (++st == kStages) {
+                    st = 0;
+                    ph ^= 1u;
                 }
             }
         }
@@ -764,74 +807,99 @@ __global__ void __launch_bounds__(kThreads, 1) k_panel_tf32x3(PanelArgs a) {
                 mbar_wait(saddr(&ctl.full[q % kStages]), (uint32_t)((q / kStages) & 1), &no_abort);
             }
         }
-    } else if (warp == kMmaWarp) {
+    } else if (warp == kMmaWarp || warp == kMmaWarp2) {
         // ------------------------------------------------------------ MMA issue
         // a.pair (default kPair) consecutive k-steps of a tile accumulate in
-        // one buffer before the drain adds it into the compensated pair
-        uint32_t st = 0, ph = 0, buf = 0, bph = 0;
-        int in_group = 0, gflags = 0;
-        if (lane == 0) {
-            bool ok = !dead;
-            while (ok) {
-                if (!mbar_wait(saddr(&ctl.full[st]), ph, &ctl.abort, a.wait_ns)) {
-                    fail(ctl, a.status);
-                    break;
-                }
-                tc_fence_after();
-                const int32_t tile = ctl.smeta_t[st], flags = ctl.smeta_f[st];
-                if (in_group == 0 && !mbar_wait(saddr(&ctl.acce[buf]), bph ^ 1u, &ctl.abort, a.wait_ns)) {
-                    fail(ctl, a.status);
-                    break;
-                }
-                tc_fence_after();
-                if (flags & kDone) {
-                    ctl.ameta_t[buf] = 0;
-                    ctl.ameta_f[buf] = kDone;
-                    mma_commit(saddr(&ctl.accf[buf]));
-                    mbar_arrive(saddr(&ctl.accf[buf]));
-                    break;
-                }
-                const uint32_t base = saddr(stages + st * kStageBytes);
-                const uint32_t acc = tmem + buf * 128;
-#pragma unroll
-                for (int kk = 0; kk < 3; ++kk) {
-                    const uint64_t ahi = sdesc(base + kk * 256, 128, kGroupStride);
-                    const uint64_t alo = sdesc(base + kGroup + kk * 256, 128, kGroupStride);
-                    const uint64_t bhi = sdesc(base + kOperand + kk * 256, 128, kGroupStride);
-                    const uint64_t blo = sdesc(base + kOperand + kGroup + kk * 256, 128, kGroupStride);
-                    mma_tf32(acc, alo, bhi, in_group > 0 || kk > 0);
-                    mma_tf32(acc, ahi, blo, 1);
-                    mma_tf32(acc, ahi, bhi, 1);
-                }
-                mma_commit(saddr(&ctl.empty[st]));
-                gflags |= flags & kFirst;
-                if ((flags & kLast) || in_group + 1 == a.pair) {
-                    ctl.ameta_t[buf] = tile;
-                    ctl.ameta_f[buf] = gflags | (flags & kLast);
-                    mma_commit(saddr(&ctl.accf[buf]));
-                    mbar_arrive(saddr(&ctl.accf[buf]));
-                    in_group = 0;
-                    gflags = 0;
-                    buf ^= 1u;
-                    if (buf == 0) bph ^= 1u;
-                } else {
-                    ++in_group;
-                }
-                if (++st == kStages) {
-                    st = 0;
-                    ph ^= 1u;
-                }
+        // one buffer, a group, before the drain adds it into the compensated
+        // pair.  Two warps take the groups in turn, an elected lane issuing:
+        // one warp's waits, issue and commits are a chain of about 1,000 cycles
+        // a k-step, of which the tensor core needs 600.
+        const int mine = warp == kMmaWarp2;
+        const int chunks = (a.s + 7) / 8;  // of 8 terms of k; the slots' rest is zeros
+        // low words of the stages' descriptors in 16-byte units, over lbo = 128 bytes
+        const uint32_t desc0 = ((saddr(stages) & 0x3FFFFu) >> 4) | ((128u >> 4) << 16);
+        uint32_t step = 0, group = 0;      // of all tiles so far
+        uint32_t rs = 0, rph = 0;
+        bool ok = !dead;
+        while (ok) {
+            if (!__all_sync(0xffffffffu, mbar_wait(saddr(&ctl.rec_full[rs]), rph, &ctl.abort, a.wait_ns))) {
+                if (lane == 0) fail(ctl, a.status);
+                break;
             }
-            // every MMA issued has completed before the tensor memory is freed
-            mma_commit(saddr(&ctl.fin));
-            if (!mbar_wait(saddr(&ctl.fin), 0, &no_abort)) fail(ctl, a.status);
+            const int32_t tile = ctl.rec[rs].tile;
+            const int n = tile < 0 ? 0 : (int)(ctl.rec[rs].s1 - ctl.rec[rs].s0);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(saddr(&ctl.rec_empty[rs]));
+            if (++rs == kRing) {
+                rs = 0;
+                rph ^= 1u;
+            }
+            for (int g0 = 0; ok && (g0 < n || tile < 0); g0 += a.pair) {
+                const int g1 = min(n, g0 + a.pair);
+                if ((int)(group & 1u) != mine) {
+                    // the other warp's: pass its stages in order (a barrier tells
+                    // only neighbouring phases apart)
+                    for (int s = g0; ok && s < g1; ++s) {
+                        const uint32_t at = step + (uint32_t)(s - g0), st = at % kStages;
+                        ok = __all_sync(0xffffffffu, mbar_wait(saddr(&ctl.full[st]), at / kStages & 1u, &ctl.abort,
+                                                               a.wait_ns));
+                        if (ok && lane == 0) mbar_arrive(saddr(&ctl.empty[st]));
+                    }
+                    if (!ok) {
+                        if (lane == 0) fail(ctl, a.status);
+                        break;
+                    }
+                } else {
+                    const uint32_t buf = group % kAcc, acc = tmem + buf * 128;
+                    ok = __all_sync(0xffffffffu, mbar_wait(saddr(&ctl.acce[buf]), (group / kAcc & 1u) ^ 1u, &ctl.abort,
+                                                           a.wait_ns));
+                    for (int s = g0; ok && s < g1; ++s) {
+                        const uint32_t at = step + (uint32_t)(s - g0), st = at % kStages;
+                        ok = __all_sync(0xffffffffu, mbar_wait(saddr(&ctl.full[st]), at / kStages & 1u, &ctl.abort,
+                                                               a.wait_ns));
+                        if (!ok) break;
+                        tc_fence_after();
+                        if (elect_one()) {
+                            const uint32_t ahi = desc0 + st * (kStageBytes / 16), alo = ahi + kGroup / 16;
+                            const uint32_t bhi = ahi + kOperand / 16, blo = bhi + kGroup / 16;
+#pragma unroll
+                            for (int kk = 0; kk < 3; ++kk)
+                                if (kk < chunks) {
+                                    mma_tf32(acc, sdesc(alo + kk * 16), sdesc(bhi + kk * 16), kk > 0 || s > g0);
+                                    mma_tf32(acc, sdesc(ahi + kk * 16), sdesc(blo + kk * 16), 1);
+                                    mma_tf32(acc, sdesc(ahi + kk * 16), sdesc(bhi + kk * 16), 1);
+                                }
+                            mma_commit(saddr(&ctl.empty[st]));
+                        }
+                        __syncwarp();
+                    }
+                    if (!ok) {
+                        if (lane == 0) fail(ctl, a.status);
+                        break;
+                    }
+                    if (elect_one()) {
+                        ctl.ameta_t[buf] = tile;
+                        ctl.ameta_f[buf] = tile < 0 ? kDone : (g0 == 0 ? kFirst : 0) | (g1 == n ? kLast : 0);
+                        mma_commit(saddr(&ctl.accf[buf]));
+                        mbar_arrive(saddr(&ctl.accf[buf]));
+                    }
+                    __syncwarp();
+                }
+                if (tile < 0) break;
+                step += (uint32_t)(g1 - g0);
+                ++group;
+            }
+            if (tile < 0) break;
+        }
+        // every MMA issued has completed before the tensor memory is freed
+        if (elect_one()) {
+            mma_commit(saddr(&ctl.fin[mine]));
+            if (!mbar_wait(saddr(&ctl.fin[mine]), 0, &no_abort)) fail(ctl, a.status);
         }
         __syncwarp();
     } else {
         // ------------------------------------------------------------ drain
-        const int quarter = warp & 3;
-        if ((warp - kMmaWarp - 1) / 4 == 0) drain<0>(a, ctl, tmem, quarter, lane, dead);
-        else drain<1>(a, ctl, tmem, quarter, lane, dead);
+        drain(a, ctl, tmem, warp & 3, (warp - kMmaWarp - 1) / 4, lane, dead);
     }
     tc_fence_before();
     __syncthreads();
