@@ -160,6 +160,11 @@ bsm_status ensure_globals() {
 
 size_t esize(int32_t dtype) { return dtype == BSM_FP64 ? 8 : 4; }
 
+// more than one block size
+bool mixed_sizes(const std::vector<int32_t> &v) {
+    return std::any_of(v.begin(), v.end(), [&](int32_t x) { return x != v[0]; });
+}
+
 bool same_vec(const std::vector<int32_t> &a, const std::vector<int32_t> &b) { return a == b; }
 
 // Phase marks of a multiply: CUDA events on the library stream when
@@ -1634,8 +1639,9 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
     // split paths: blocks of one tile row in their own kernel instance, unless
     // the tuning fixes the pass rows; Ozaki path: blocks of one tile column
     const bool want_groups = rprec == BSM_P_OZAKI || tune_of(rprec)[BSM_TUNE_PASS_MT] <= 0;
-    // the FP64 kernel groups small blocks by itself: no variant marks in its order
-    const int order_prec = kprec == BSM_P_FP64 && A->dtype == BSM_FP64 ? -1 : rprec;
+    // the CUDA-core kernels group small blocks by themselves: no variant marks in their order
+    const bool cores = kprec == BSM_P_FP64 || (kprec == BSM_P_FP64_DMMA && A->dtype != BSM_FP64);
+    const int order_prec = cores ? -1 : rprec;
     auto numeric_pass = [&](int64_t cb0, int64_t nitems, int64_t nprod_pass, bool whole) -> bsm_status {
         NumericArgs na{};
         na.n_items = nitems;
@@ -1655,6 +1661,7 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
         na.prec = kprec;
         na.flush_every = opts.flush_every;
         na.max_out_rows = A->max_bs_row; na.max_out_cols = B->max_bs_col;
+        na.mixed_k = mixed_sizes(A->h_col_bs);
         na.x_pack = pkA.words; na.x_pack_off = pkA.off;
         na.y_pack = pkB.words; na.y_pack_off = pkB.off;
         na.x_exp = olA.exps; na.x_line0 = olA.line0;
@@ -1932,6 +1939,7 @@ bsm_status bsm_multiply_backward(double alpha, bsm_t C, const void *dC_data, bsm
         na.dtype = C->dtype;
         na.prec = kprec;
         na.max_out_rows = OUT->max_bs_row; na.max_out_cols = OUT->max_bs_col;
+        na.mixed_k = mixed_sizes(side == 0 ? B->h_col_bs : A->h_row_bs);
         na.flush_every = opts.flush_every;
         na.x_pack = pkX.words; na.x_pack_off = pkX.off;
         na.y_pack = pkY.words; na.y_pack_off = pkY.off;
@@ -1942,7 +1950,8 @@ bsm_status bsm_multiply_backward(double alpha, bsm_t C, const void *dC_data, bsm
         int64_t *n_marked = nullptr;
         bool uses_cores = false;
         if ((st = shape_order(sc, OUT->nnzb, OUT->blk_rc, OUT->h_row_bs, OUT->h_col_bs, &item_order, nullptr, nullptr,
-                              kprec == BSM_P_FP64 && C->dtype == BSM_FP64 ? -1 : opts.prec, &uses_cores, &n_marked)))
+                              kprec == BSM_P_FP64 || (kprec == BSM_P_FP64_DMMA && C->dtype != BSM_FP64) ? -1 : opts.prec,
+                              &uses_cores, &n_marked)))
             return st;
         na.n_lane_items = n_marked;
         if (needs_plain(kprec) && uses_cores && nprod > 0) {

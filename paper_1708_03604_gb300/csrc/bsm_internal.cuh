@@ -270,6 +270,7 @@ struct NumericArgs {
     // unpacked split pieces (CUDA-core variant of the split paths)
     const float *x_plain, *y_plain;
     int32_t max_out_rows, max_out_cols;
+    int32_t mixed_k;            // the inner dimension has blocks of different sizes
     const int32_t *item_order;  // nullable: processing order of the items (grouped by block shape);
                                 // bit 31 marks the second variant of the item's shape
     const int64_t *n_lane_items;  // nullable (CUDA-core FP64 path): the last *n_lane_items items of
@@ -311,6 +312,9 @@ constexpr int kCcSmall = 0, kCcNarrow = 1, kCcWide = 2;
 // FP64 data on the CUDA cores (k_group.cu); *grid: CTAs launched
 cudaError_t launch_numeric_group(const NumericArgs &a, int build, cudaStream_t s, int *grid);
 uint32_t group_debug_bits(cudaStream_t s);
+// FP32 data on the CUDA cores (k_tile.cu)
+cudaError_t launch_numeric_tile(const NumericArgs &a, cudaStream_t s, int *grid);
+uint32_t tile_debug_bits(cudaStream_t s);
 int num_sms();
 // out[g] = number of keys below thr[g] in the ascending keys[0..n) (g < 2)
 cudaError_t launch_group_bounds(const uint32_t *keys, int64_t n, uint32_t thr0, uint32_t thr1, int64_t *out,

@@ -12,8 +12,8 @@
 //   adjoint  dB_kj = sum_i A_ik^T . dC_ij       X = A^T,    Y = dC
 //
 // Two arithmetic paths:
-//   * CUDA cores: FP64 FMA for FP64 data (FP32 FMA with an FP64 running sum
-//     for FP32 data); one lane owns a fixed set of output elements.
+//   * CUDA cores: FP64 FMA; one lane owns a fixed set of output elements (the
+//     plain FP64 path is in k_group.cu, FP32 data in k_tile.cu).
 //   * Tensor cores (mma.sync m16n8k8 TF32 / m16n8k16 BF16): operands were
 //     split beforehand into 2 or 3 narrow pieces (hi, lo[, lo2]) and packed
 //     in mma fragment order; the cross products of the pieces accumulate in
@@ -35,26 +35,26 @@ constexpr int kWarpsPerCta = 4;             // default warps per CTA
 constexpr int kThreadsNum = kWarpsPerCta * 32;
 
 // =====================================================================
-// CUDA-core path
+// FP64 FMA on the CUDA cores, a warp or a lane per output block: the small
+// blocks of the FP64 tensor-core and Ozaki paths (BSM_P_FP64 has k_group.cu,
+// FP32 data k_tile.cu)
 // =====================================================================
-template <typename T, int Q>
+template <int Q>
 __device__ __forceinline__ void cc_item(const NumericArgs &a, int64_t q, int lane) {
-    const T *__restrict__ X = static_cast<const T *>(a.x_data);
-    const T *__restrict__ Y = static_cast<const T *>(a.y_data);
-    T *__restrict__ O = static_cast<T *>(a.out_data);
+    const double *__restrict__ X = static_cast<const double *>(a.x_data);
+    const double *__restrict__ Y = static_cast<const double *>(a.y_data);
+    double *__restrict__ O = static_cast<double *>(a.out_data);
     const int32_t orc = a.out_blk_rc[q];
     const int R = rc_rows(orc), S = rc_cols(orc);
     const int RS = R * S;
     const int64_t out_off = a.out_blk_off[q];
     const int64_t p0 = a.seg_ptr[q], p1 = a.seg_ptr[q + 1];
     const int64_t old = (a.beta != 0.0 && a.old_off) ? a.old_off[q] : -1;
-    const T *OLD = static_cast<const T *>(a.old_data);
-    const int F = a.flush_every > 0 ? a.flush_every : 1;
+    const double *OLD = static_cast<const double *>(a.old_data);
 
     for (int e0 = 0; e0 < RS; e0 += 32 * Q) {
         int rr[Q], ss[Q];
         double acc[Q];
-        T acc_n[Q];
 #pragma unroll
         for (int u = 0; u < Q; ++u) {
             const int e = e0 + lane + 32 * u;
@@ -62,13 +62,11 @@ __device__ __forceinline__ void cc_item(const NumericArgs &a, int64_t q, int lan
             rr[u] = v ? e / S : 0;
             ss[u] = v ? e % S : 0;
             acc[u] = 0.0;
-            acc_n[u] = T(0);
         }
-        int since = 0;
         for (int64_t p = p0; p < p1; ++p) {
             const int32_t ix = a.px[p], iy = a.py[p];
-            const T *xb = X + a.x_blk_off[ix];
-            const T *yb = Y + a.y_blk_off[iy];
+            const double *xb = X + a.x_blk_off[ix];
+            const double *yb = Y + a.y_blk_off[iy];
             const int32_t xrc = a.x_blk_rc[ix];
             const int Tn = a.x_trans ? rc_rows(xrc) : rc_cols(xrc);
             const int xs_r = a.x_trans ? 1 : Tn, xs_t = a.x_trans ? R : 1;
@@ -82,19 +80,9 @@ __device__ __forceinline__ void cc_item(const NumericArgs &a, int64_t q, int lan
             for (int t = 0; t < Tn; ++t) {
 #pragma unroll
                 for (int u = 0; u < Q; ++u) {
-                    const T xv = __ldg(xb + xo[u] + t * xs_t);
-                    const T yv = __ldg(yb + t * ys_t + yo[u]);
-                    acc_n[u] = fma(xv, yv, acc_n[u]);
-                }
-            }
-            if constexpr (sizeof(T) == 4) {
-                if (++since == F) {
-                    since = 0;
-#pragma unroll
-                    for (int u = 0; u < Q; ++u) {
-                        acc[u] += (double)acc_n[u];
-                        acc_n[u] = T(0);
-                    }
+                    const double xv = __ldg(xb + xo[u] + t * xs_t);
+                    const double yv = __ldg(yb + t * ys_t + yo[u]);
+                    acc[u] = fma(xv, yv, acc[u]);
                 }
             }
         }
@@ -102,62 +90,34 @@ __device__ __forceinline__ void cc_item(const NumericArgs &a, int64_t q, int lan
         for (int u = 0; u < Q; ++u) {
             const int e = e0 + lane + 32 * u;
             if (e < RS) {
-                double v = (sizeof(T) == 8) ? (double)acc_n[u] : acc[u] + (double)acc_n[u];
+                double v = acc[u];
                 v = a.alpha * v;
-                if (old >= 0) v = fma(a.beta, (double)OLD[old + e], v);
-                O[out_off + e] = (T)v;
+                if (old >= 0) v = fma(a.beta, OLD[old + e], v);
+                O[out_off + e] = v;
             }
         }
     }
 }
 
-// Builds of the CUDA-core kernel (the widest element-per-lane template sets
-// the register count, and with it how many warps an SM holds):
-//   kCcSmall  every output block has at most 16 elements: one element per lane
-//             at most (72 registers)
-//   kCcNarrow up to 9 elements per lane per pass, more passes over the
-//             products for larger blocks (128 registers)
-//   kCcWide   up to 24 elements per lane per pass (253 registers)
-template <typename T, int BUILD>
+// up to 9 elements per lane per pass, more passes over the products for larger blocks
 __device__ __forceinline__ void cc_dispatch(const NumericArgs &a, int64_t q, int lane) {
-    if constexpr (BUILD == kCcSmall) {
-        cc_item<T, 1>(a, q, lane);
-        return;
-    }
     const int32_t orc = a.out_blk_rc[q];
-    const int RS = rc_rows(orc) * rc_cols(orc);
-    const int need = (RS + 31) >> 5;
-    if constexpr (BUILD == kCcNarrow) {
-        if (need <= 1) cc_item<T, 1>(a, q, lane);
-        else if (need <= 2) cc_item<T, 2>(a, q, lane);
-        else if (need <= 3) cc_item<T, 3>(a, q, lane);
-        else if (need <= 4) cc_item<T, 4>(a, q, lane);
-        else if (need <= 6) cc_item<T, 6>(a, q, lane);
-        else cc_item<T, 9>(a, q, lane);
-        return;
-    }
-    if (need <= 1) cc_item<T, 1>(a, q, lane);
-    else if (need <= 2) cc_item<T, 2>(a, q, lane);
-    else if (need <= 3) cc_item<T, 3>(a, q, lane);
-    else if (need <= 4) cc_item<T, 4>(a, q, lane);
-    else if (need <= 6) cc_item<T, 6>(a, q, lane);
-    else if (need <= 8) cc_item<T, 8>(a, q, lane);
-    else if (need <= 10) cc_item<T, 10>(a, q, lane);
-    else if (need <= 12) cc_item<T, 12>(a, q, lane);
-    else if (need <= 14) cc_item<T, 14>(a, q, lane);
-    else if (need <= 17) cc_item<T, 17>(a, q, lane);
-    else if (need <= 20) cc_item<T, 20>(a, q, lane);
-    else cc_item<T, 24>(a, q, lane);
+    const int need = (rc_rows(orc) * rc_cols(orc) + 31) >> 5;
+    if (need <= 1) cc_item<1>(a, q, lane);
+    else if (need <= 2) cc_item<2>(a, q, lane);
+    else if (need <= 3) cc_item<3>(a, q, lane);
+    else if (need <= 4) cc_item<4>(a, q, lane);
+    else if (need <= 6) cc_item<6>(a, q, lane);
+    else cc_item<9>(a, q, lane);
 }
 
 // Tiny output blocks (at most 16 elements): one lane owns a whole block, so a
 // warp advances 32 blocks at once instead of leaving most lanes idle.
-template <typename T>
 __device__ __forceinline__ void cc_lane_item(const NumericArgs &a, int64_t q) {
     constexpr int L = 16;
-    const T *__restrict__ X = static_cast<const T *>(a.x_data);
-    const T *__restrict__ Y = static_cast<const T *>(a.y_data);
-    T *__restrict__ O = static_cast<T *>(a.out_data);
+    const double *__restrict__ X = static_cast<const double *>(a.x_data);
+    const double *__restrict__ Y = static_cast<const double *>(a.y_data);
+    double *__restrict__ O = static_cast<double *>(a.out_data);
     const int32_t orc = a.out_blk_rc[q];
     const int R = rc_rows(orc), S = rc_cols(orc);
     const int RS = R * S;
@@ -165,16 +125,14 @@ __device__ __forceinline__ void cc_lane_item(const NumericArgs &a, int64_t q) {
     const int64_t p0 = a.seg_ptr[q], p1 = a.seg_ptr[q + 1];
     const int64_t old = (a.beta != 0.0 && a.old_off) ? a.old_off[q] : -1;
     double acc[L];
-    T acc_n[L];
 #pragma unroll
     for (int e = 0; e < L; ++e) {
         acc[e] = 0.0;
-        acc_n[e] = T(0);
     }
     for (int64_t p = p0; p < p1; ++p) {
         const int32_t ix = a.px[p], iy = a.py[p];
-        const T *xb = X + a.x_blk_off[ix];
-        const T *yb = Y + a.y_blk_off[iy];
+        const double *xb = X + a.x_blk_off[ix];
+        const double *yb = Y + a.y_blk_off[iy];
         const int32_t xrc = a.x_blk_rc[ix];
         const int Tn = a.x_trans ? rc_rows(xrc) : rc_cols(xrc);
         const int xs_r = a.x_trans ? 1 : Tn, xs_t = a.x_trans ? R : 1;
@@ -184,59 +142,50 @@ __device__ __forceinline__ void cc_lane_item(const NumericArgs &a, int64_t q) {
             for (int e = 0; e < L; ++e) {
                 if (e < RS) {
                     const int r = e / S, c = e - r * S;
-                    acc_n[e] = fma(__ldg(xb + r * xs_r + t * xs_t), __ldg(yb + t * ys_t + c * ys_s), acc_n[e]);
+                    acc[e] = fma(__ldg(xb + r * xs_r + t * xs_t), __ldg(yb + t * ys_t + c * ys_s), acc[e]);
                 }
             }
         }
-        if constexpr (sizeof(T) == 4) {
-#pragma unroll
-            for (int e = 0; e < L; ++e) {
-                acc[e] += (double)acc_n[e];
-                acc_n[e] = T(0);
-            }
-        }
     }
-    const T *OLD = static_cast<const T *>(a.old_data);
+    const double *OLD = static_cast<const double *>(a.old_data);
 #pragma unroll
     for (int e = 0; e < L; ++e) {
         if (e < RS) {
-            double v = (sizeof(T) == 8) ? (double)acc_n[e] : acc[e];
+            double v = acc[e];
             v = a.alpha * v;
-            if (old >= 0) v = fma(a.beta, (double)OLD[old + e], v);
-            O[out_off + e] = (T)v;
+            if (old >= 0) v = fma(a.beta, OLD[old + e], v);
+            O[out_off + e] = v;
         }
     }
 }
 
 // Fixed shapes of the lane-per-block mode: column t of the X block and row t
 // of the Y block are loaded once per k and applied as a rank-1 update.
-template <typename T, int R, int S>
+template <int R, int S>
 __device__ __forceinline__ void cc_lane_fixed(const NumericArgs &a, int64_t q) {
-    const T *__restrict__ X = static_cast<const T *>(a.x_data);
-    const T *__restrict__ Y = static_cast<const T *>(a.y_data);
-    T *__restrict__ O = static_cast<T *>(a.out_data);
+    const double *__restrict__ X = static_cast<const double *>(a.x_data);
+    const double *__restrict__ Y = static_cast<const double *>(a.y_data);
+    double *__restrict__ O = static_cast<double *>(a.out_data);
     const int64_t out_off = a.out_blk_off[q];
     const int64_t p0 = a.seg_ptr[q], p1 = a.seg_ptr[q + 1];
     const int64_t old = (a.beta != 0.0 && a.old_off) ? a.old_off[q] : -1;
     double acc[R][S];
-    T acc_n[R][S];
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int c = 0; c < S; ++c) {
             acc[r][c] = 0.0;
-            acc_n[r][c] = T(0);
         }
     for (int64_t p = p0; p < p1; ++p) {
         const int32_t ix = a.px[p], iy = a.py[p];
-        const T *xb = X + a.x_blk_off[ix];
-        const T *yb = Y + a.y_blk_off[iy];
+        const double *xb = X + a.x_blk_off[ix];
+        const double *yb = Y + a.y_blk_off[iy];
         const int32_t xrc = a.x_blk_rc[ix];
         const int Tn = a.x_trans ? rc_rows(xrc) : rc_cols(xrc);
         const int xs_r = a.x_trans ? 1 : Tn, xs_t = a.x_trans ? R : 1;
         const int ys_t = a.y_trans ? 1 : S, ys_s = a.y_trans ? Tn : 1;
         for (int t = 0; t < Tn; ++t) {
-            T xv[R], yv[S];
+            double xv[R], yv[S];
 #pragma unroll
             for (int r = 0; r < R; ++r) xv[r] = __ldg(xb + r * xs_r + t * xs_t);
 #pragma unroll
@@ -244,87 +193,37 @@ __device__ __forceinline__ void cc_lane_fixed(const NumericArgs &a, int64_t q) {
 #pragma unroll
             for (int r = 0; r < R; ++r)
 #pragma unroll
-                for (int c = 0; c < S; ++c) acc_n[r][c] = fma(xv[r], yv[c], acc_n[r][c]);
-        }
-        if constexpr (sizeof(T) == 4) {
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-#pragma unroll
-                for (int c = 0; c < S; ++c) {
-                    acc[r][c] += (double)acc_n[r][c];
-                    acc_n[r][c] = T(0);
-                }
+                for (int c = 0; c < S; ++c) acc[r][c] = fma(xv[r], yv[c], acc[r][c]);
         }
     }
-    const T *OLD = static_cast<const T *>(a.old_data);
+    const double *OLD = static_cast<const double *>(a.old_data);
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int c = 0; c < S; ++c) {
             const int e = r * S + c;
-            double v = (sizeof(T) == 8) ? (double)acc_n[r][c] : acc[r][c];
+            double v = acc[r][c];
             v = a.alpha * v;
-            if (old >= 0) v = fma(a.beta, (double)OLD[old + e], v);
-            O[out_off + e] = (T)v;
+            if (old >= 0) v = fma(a.beta, OLD[old + e], v);
+            O[out_off + e] = v;
         }
 }
 
-template <typename T, int BUILD = kCcWide>
 __device__ __forceinline__ void cc_lane_dispatch(const NumericArgs &a, int64_t q) {
     const int32_t orc = a.out_blk_rc[q];
-    if constexpr (BUILD == kCcSmall) {
-        switch ((rc_rows(orc) << 8) | rc_cols(orc)) {
-            case 0x101: cc_lane_fixed<T, 1, 1>(a, q); break;
-            case 0x104: cc_lane_fixed<T, 1, 4>(a, q); break;
-            case 0x401: cc_lane_fixed<T, 4, 1>(a, q); break;
-            case 0x404: cc_lane_fixed<T, 4, 4>(a, q); break;
-            case 0x202: cc_lane_fixed<T, 2, 2>(a, q); break;
-            default: cc_lane_item<T>(a, q); break;
-        }
-        return;
-    }
     switch ((rc_rows(orc) << 8) | rc_cols(orc)) {
-        case 0x101: cc_lane_fixed<T, 1, 1>(a, q); break;
-        case 0x102: cc_lane_fixed<T, 1, 2>(a, q); break;
-        case 0x201: cc_lane_fixed<T, 2, 1>(a, q); break;
-        case 0x202: cc_lane_fixed<T, 2, 2>(a, q); break;
-        case 0x104: cc_lane_fixed<T, 1, 4>(a, q); break;
-        case 0x401: cc_lane_fixed<T, 4, 1>(a, q); break;
-        case 0x204: cc_lane_fixed<T, 2, 4>(a, q); break;
-        case 0x402: cc_lane_fixed<T, 4, 2>(a, q); break;
-        case 0x404: cc_lane_fixed<T, 4, 4>(a, q); break;
-        case 0x505: cc_lane_fixed<T, 5, 5>(a, q); break;
-        case 0x606: cc_lane_fixed<T, 6, 6>(a, q); break;
-        default: cc_lane_item<T>(a, q); break;
-    }
-}
-
-template <typename T, int BUILD>
-__global__ void __launch_bounds__(kThreadsNum) k_numeric_cc(NumericArgs a) {
-    const int lane = threadIdx.x & 31;
-    if (a.status && *a.status != 0) return;
-    unsigned long long *ctr = a.work_counter;
-    // items [0, n0): a warp each; items [n0, n_items): marked tiny blocks, 32 per ticket
-    const int64_t n_lane = a.n_lane_items ? *a.n_lane_items : 0;
-    const int64_t n0 = a.n_items - n_lane;
-    const int64_t tickets = n0 + (n_lane + 31) / 32;
-    while (true) {
-        int64_t t = 0;
-        if (lane == 0) t = (int64_t)atomicAdd(ctr, 1ull);
-        t = __shfl_sync(0xffffffffu, t, 0);
-        if (t >= tickets) break;
-        if (t < n0) {
-            int64_t q = t;
-            if (a.item_order) q = (int64_t)((uint32_t)a.item_order[q] & 0x7fffffffu);
-            BSM_DBG_WARP_SKIP(a, q, lane)
-            cc_dispatch<T, BUILD>(a, q, lane);
-        } else {
-            const int64_t idx = n0 + (t - n0) * 32 + lane;
-            if (idx < a.n_items) {
-                const int64_t q = (int64_t)((uint32_t)a.item_order[idx] & 0x7fffffffu);
-                if (BSM_DBG_LANE_OK(a, q)) cc_lane_dispatch<T, BUILD>(a, q);
-            }
-        }
+        case 0x101: cc_lane_fixed<1, 1>(a, q); break;
+        case 0x102: cc_lane_fixed<1, 2>(a, q); break;
+        case 0x201: cc_lane_fixed<2, 1>(a, q); break;
+        case 0x202: cc_lane_fixed<2, 2>(a, q); break;
+        case 0x104: cc_lane_fixed<1, 4>(a, q); break;
+        case 0x401: cc_lane_fixed<4, 1>(a, q); break;
+        case 0x204: cc_lane_fixed<2, 4>(a, q); break;
+        case 0x402: cc_lane_fixed<4, 2>(a, q); break;
+        case 0x404: cc_lane_fixed<4, 4>(a, q); break;
+        case 0x505: cc_lane_fixed<5, 5>(a, q); break;
+        case 0x606: cc_lane_fixed<6, 6>(a, q); break;
+        default: cc_lane_item(a, q); break;
     }
 }
 
@@ -453,12 +352,12 @@ __global__ void __launch_bounds__(kThreadsNum) k_numeric_dmma(NumericArgs a) {
             BSM_DBG_WARP_SKIP(a, q, lane)
             const int32_t orc = a.out_blk_rc[q];
             if (rc_rows(orc) >= 8 && rc_cols(orc) >= 8) dmma_item(a, q, lane);
-            else cc_dispatch<double, kCcNarrow>(a, q, lane);
+            else cc_dispatch(a, q, lane);
         } else {
             const int64_t idx = n0 + (t - n0) * 32 + lane;
             if (idx < a.n_items) {
                 const int64_t q = (int64_t)((uint32_t)a.item_order[idx] & 0x7fffffffu);
-                if (BSM_DBG_LANE_OK(a, q)) cc_lane_dispatch<double, kCcNarrow>(a, q);
+                if (BSM_DBG_LANE_OK(a, q)) cc_lane_dispatch(a, q);
             }
         }
     }
@@ -1345,7 +1244,7 @@ __global__ void __launch_bounds__(kThreadsNum) k_numeric_oz_lane(NumericArgs a) 
         const int64_t idx = lane0 + t * 32 + lane;
         if (idx < a.n_items) {
             const int64_t q = (int64_t)((uint32_t)a.item_order[idx] & 0x7fffffffu);
-            if (BSM_DBG_LANE_OK(a, q)) cc_lane_dispatch<double>(a, q);
+            if (BSM_DBG_LANE_OK(a, q)) cc_lane_dispatch(a, q);
         }
     }
 }
@@ -1679,13 +1578,6 @@ int persistent_grid(K kernel, int64_t n_items, size_t smem = 0, int threads = kT
     return (int)g;
 }
 
-template <typename T, int BUILD>
-int launch_cc(const NumericArgs &a, cudaStream_t s) {
-    const int g = persistent_grid(k_numeric_cc<T, BUILD>, a.n_items, 0, kThreadsNum, a.ctas_per_sm);
-    k_numeric_cc<T, BUILD><<<g, kThreadsNum, 0, s>>>(a);
-    return g;
-}
-
 template <int MAXN>
 cudaError_t launch_oz(const NumericArgs &a, cudaStream_t s, int threads, int *grid) {
     const size_t smem = sizeof(uint32_t) * (size_t)oz_ring_words_per_warp<MAXN>() * (threads / 32);
@@ -1833,9 +1725,7 @@ cudaError_t launch_numeric(const NumericArgs &args, cudaStream_t s, NumericLaunc
         if (a.dtype == BSM_FP64) {
             e = launch_numeric_group(a, build, s, &grid);
         } else {
-            if (build == kCcSmall) grid = launch_cc<float, kCcSmall>(a, s);
-            else if (build == kCcNarrow) grid = launch_cc<float, kCcNarrow>(a, s);
-            else grid = launch_cc<float, kCcWide>(a, s);
+            e = launch_numeric_tile(a, s, &grid);
         }
         li = NumericLaunch{BSM_K_FP64_CORES, build, kThreadsNum, grid, 0, 0};
     } else {
@@ -1851,7 +1741,7 @@ cudaError_t launch_numeric(const NumericArgs &args, cudaStream_t s, NumericLaunc
     return cudaGetLastError();
 }
 
-uint32_t numeric_debug_bits(cudaStream_t s) { return read_debug_bits(s) | group_debug_bits(s); }
+uint32_t numeric_debug_bits(cudaStream_t s) { return read_debug_bits(s) | group_debug_bits(s) | tile_debug_bits(s); }
 
 cudaError_t launch_split_plain(const bsm_mat *M, int prec, float *out, cudaStream_t s) {
     if (M->data_len == 0) return cudaSuccess;

@@ -1,9 +1,10 @@
-"""The FP64 kernel's lane groups (GPU): output blocks of every layout the
+"""The CUDA-core kernels' lane groups (GPU): output blocks of every layout the
 kernel chooses from (a warp per block, several blocks per warp in row- or
 column-keeping groups, several passes over large blocks), with enough blocks
 that small ones share a warp.  Every element is one chain of FP64 fused
 multiply-adds in ascending k whatever the layout, so the builds (which choose
-different layouts) must agree bit for bit; against the oracle 1e-12."""
+different layouts) must agree bit for bit; against the oracle 1e-12.  FP32
+data runs register tiles in lane groups, checked against FP64 data."""
 import numpy as np
 import pytest
 
@@ -73,6 +74,55 @@ def test_layouts_agree_and_match_oracle(bsm, oracle, sizes):
     c, = _with_builds(bsm, merged)
     ref = oracle.multiply(-0.75, Ah, Bh, eps=0.9, beta=0.5, Cold=C0)
     assert rel_fro(c, ref.C.data) <= 1e-12
+
+
+FP32_SHAPES = [(1,), (3,), (4,), (5,), (8,), (13,), (17,), (24,), (25,), (33,), (4, 1), (5, 13, 23), (3, 7, 16, 32)]
+
+
+@pytest.mark.parametrize("sizes", FP32_SHAPES, ids=lambda s: "_".join(map(str, s)))
+def test_fp32_tiles_within_their_bound(bsm, sizes):
+    """FP32 data: one FP32 chain of fused multiply-adds per product and element, the products added in FP64 in
+    order.  Every element within the bound of that: k roundings of 2^-24 of the magnitude in the longest product
+    and one of the result (doubled: 2^-23), against FP64 data of the same values; the adjoints within 1e-5."""
+    import torch
+    nb = 150 if max(sizes) < 24 else 100
+    bs = I.mixed_sizes(nb, sizes, [1.0 / len(sizes)] * len(sizes), seed=5)
+    Ah, Bh = random_bcsr(bs, bs, 0.12, seed=61, dtype=np.float32), random_bcsr(bs, bs, 0.12, seed=62, dtype=np.float32)
+    A, B = bsm.Matrix.from_host(Ah), bsm.Matrix.from_host(Bh)
+    A64, B64 = bsm.Matrix.from_host(Ah.astype(np.float64)), bsm.Matrix.from_host(Bh.astype(np.float64))
+    C, C64 = bsm.multiply(1.0, A, B), bsm.multiply(1.0, A64, B64)
+    c, c64 = C.data_host().astype(np.float64), C64.data_host()
+    # magnitude of every element's terms, from the absolute values
+    absA, absB = (bsm.Matrix.from_host(I.BCSR(*(list(vars(X).values())[:5]), np.abs(X.data).astype(np.float64)))
+                  for X in (Ah, Bh))
+    mag = bsm.multiply(1.0, absA, absB).data_host()
+    assert (np.abs(c - c64) <= (max(sizes) + 2) * 2.0 ** -23 * mag).all()
+    g64 = torch.linspace(-1.0, 1.0, C.info().data_len, dtype=torch.float64, device="cuda")
+    g = g64.float()
+    got, ref = [], []
+    for out, Cx, Ax, Bx, gx in ((got, C, A, B, g), (ref, C64, A64, B64, g.double())):
+        dA, dB = (torch.full((len(X.data),), np.nan, dtype=gx.dtype, device="cuda") for X in (Ah, Bh))
+        bsm.multiply_backward(-0.5, Cx, gx, Ax, Bx, dA, dB)
+        out += [dA.double().cpu().numpy(), dB.double().cpu().numpy()]
+    for x, y in zip(got, ref):
+        assert rel_fro(x, y) <= 1e-5
+
+
+def test_fp32_old_blocks_zero_and_non_finite(bsm):
+    """Old blocks merged with beta, zero partial sums (converted the usual way) and infinities, against FP64 data."""
+    bs = I.mixed_sizes(120, (5, 8, 23), (0.4, 0.3, 0.3), seed=9)
+    Ah, Bh = random_bcsr(bs, bs, 0.1, seed=71), random_bcsr(bs, bs, 0.1, seed=72)
+    C0 = random_bcsr(bs, bs, 0.2, seed=73)
+    Ah.data[: len(Ah.data) // 3] = 0.0
+    Bh.data[-1] = np.inf
+    f = np.float32
+    Ah.data, Bh.data, C0.data = (X.data.astype(f).astype(np.float64) for X in (Ah, Bh, C0))
+    want = bsm.multiply(0.5, *(bsm.Matrix.from_host(X) for X in (Ah, Bh)), 2.0, bsm.Matrix.from_host(C0)).data_host()
+    got = bsm.multiply(0.5, *(bsm.Matrix.from_host(X.astype(f)) for X in (Ah, Bh)), 2.0,
+                       bsm.Matrix.from_host(C0.astype(f))).data_host().astype(np.float64)
+    fin = np.isfinite(want)
+    np.testing.assert_array_equal(np.isfinite(got), fin)
+    assert rel_fro(got[fin], want[fin]) <= 1e-5
 
 
 def test_non_finite_values_stay_in_their_rows(bsm):
