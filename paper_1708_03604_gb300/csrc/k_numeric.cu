@@ -684,201 +684,67 @@ __device__ __forceinline__ void tc_item(const NumericArgs &a, int64_t q, int lan
     }
 }
 
-// Tiny output blocks (at most 16 elements) on the split paths: one lane owns
-// a whole block and multiplies the same narrow pieces with FP32 FMA on CUDA
-// cores (a product of two TF32 or BF16 pieces is exact in FP32), FP32 sum
-// inside a block product, the same compensated (or FP64) sum across products.
-// A 16 x 8 MMA tile would be almost all padding for such blocks.
+// Tiny output blocks (at most 16 elements, 5 x 5 on request) on the split
+// paths: the same narrow pieces multiplied with FP32 FMA on CUDA cores (a
+// product of two TF32 or BF16 pieces is exact in FP32), FP32 sum inside a block
+// product, the same compensated (or FP64) sum across products.  A 16 x 8 MMA
+// tile would be almost all padding for such blocks.  One lane owns one element:
+// a lane per block leaves a few blocks with long product lists to a few warps
+// (2,700 blocks of ragged sizes 1..40: 7.0 ms).
 template <int PREC, bool FF>
-__device__ __forceinline__ void cs_lane_item(const NumericArgs &a, int64_t q) {
+__device__ __forceinline__ void cs_element(const NumericArgs &a, int64_t q, int e) {
     constexpr int NP = PrecTraits<PREC>::NP;
-    constexpr int L = 16;
-    const float *__restrict__ X = a.x_plain;
-    const float *__restrict__ Y = a.y_plain;
     const int32_t orc = a.out_blk_rc[q];
-    const int R = rc_rows(orc), S = rc_cols(orc);
-    const int RS = R * S;
-    const int64_t out_off = a.out_blk_off[q];
-    const int64_t p0 = a.seg_ptr[q], p1 = a.seg_ptr[q + 1];
+    const int R = rc_rows(orc), S = rc_cols(orc), r = e / S, c = e - r * S;
+    const int64_t p1 = a.seg_ptr[q + 1];
     const int64_t old = (a.beta != 0.0 && a.old_off) ? a.old_off[q] : -1;
     const int F = a.flush_every > 0 ? a.flush_every : (a.flush_every < 0 ? -a.flush_every : 1);
-    float acc[L], shi[FF ? L : 1], slo[FF ? L : 1];
-    double s64[FF ? 1 : L];
-#pragma unroll
-    for (int e = 0; e < L; ++e) {
-        acc[e] = 0.f;
-        if constexpr (FF) {
-            shi[e] = 0.f;
-            slo[e] = 0.f;
-        } else {
-            s64[e] = 0.0;
-        }
-    }
+    float acc = 0.f, shi = 0.f, slo = 0.f;
+    double s64 = 0.0;
     int since = 0;
-    for (int64_t p = p0; p < p1; ++p) {
+    for (int64_t p = a.seg_ptr[q]; p < p1; ++p) {
         const int32_t ix = a.px[p], iy = a.py[p];
-        const float *xb = X + a.x_blk_off[ix] * NP;
-        const float *yb = Y + a.y_blk_off[iy] * NP;
         const int32_t xrc = a.x_blk_rc[ix];
         const int Tn = a.x_trans ? rc_rows(xrc) : rc_cols(xrc);
-        const int xs_r = a.x_trans ? 1 : Tn, xs_t = a.x_trans ? R : 1;
-        const int ys_t = a.y_trans ? 1 : S, ys_s = a.y_trans ? Tn : 1;
+        const int xs_t = a.x_trans ? R : 1, ys_t = a.y_trans ? 1 : S;
+        const float *xe = a.x_plain + (a.x_blk_off[ix] + r * (a.x_trans ? 1 : Tn)) * NP;
+        const float *ye = a.y_plain + (a.y_blk_off[iy] + c * (a.y_trans ? Tn : 1)) * NP;
+#pragma unroll 4
         for (int t = 0; t < Tn; ++t) {
-#pragma unroll
-            for (int e = 0; e < L; ++e) {
-                if (e < RS) {
-                    const int r = e / S, c = e - r * S;
-                    const float *xe = xb + (int64_t)(r * xs_r + t * xs_t) * NP;
-                    const float *ye = yb + (int64_t)(t * ys_t + c * ys_s) * NP;
-                    if constexpr (NP == 2) {
-                        const float2 xv = __ldg(reinterpret_cast<const float2 *>(xe));
-                        const float2 yv = __ldg(reinterpret_cast<const float2 *>(ye));
-                        acc[e] = fmaf(xv.y, yv.x, acc[e]);
-                        acc[e] = fmaf(xv.x, yv.y, acc[e]);
-                        acc[e] = fmaf(xv.x, yv.x, acc[e]);
-                    } else {
-                        const float x0 = __ldg(xe), x1 = __ldg(xe + 1), x2 = __ldg(xe + 2);
-                        const float y0 = __ldg(ye), y1 = __ldg(ye + 1), y2 = __ldg(ye + 2);
-                        acc[e] = fmaf(x2, y0, acc[e]);
-                        acc[e] = fmaf(x1, y1, acc[e]);
-                        acc[e] = fmaf(x0, y2, acc[e]);
-                        acc[e] = fmaf(x1, y0, acc[e]);
-                        acc[e] = fmaf(x0, y1, acc[e]);
-                        acc[e] = fmaf(x0, y0, acc[e]);
-                    }
-                }
+            if constexpr (NP == 2) {
+                const float2 xv = __ldg(reinterpret_cast<const float2 *>(xe + (int64_t)t * xs_t * NP));
+                const float2 yv = __ldg(reinterpret_cast<const float2 *>(ye + (int64_t)t * ys_t * NP));
+                acc = fmaf(xv.y, yv.x, acc);
+                acc = fmaf(xv.x, yv.y, acc);
+                acc = fmaf(xv.x, yv.x, acc);
+            } else {
+                const float *xt = xe + (int64_t)t * xs_t * NP, *yt = ye + (int64_t)t * ys_t * NP;
+                const float x0 = __ldg(xt), x1 = __ldg(xt + 1), x2 = __ldg(xt + 2);
+                const float y0 = __ldg(yt), y1 = __ldg(yt + 1), y2 = __ldg(yt + 2);
+                acc = fmaf(x2, y0, acc);
+                acc = fmaf(x1, y1, acc);
+                acc = fmaf(x0, y2, acc);
+                acc = fmaf(x1, y0, acc);
+                acc = fmaf(x0, y1, acc);
+                acc = fmaf(x0, y0, acc);
             }
         }
         if (++since == F) {
             since = 0;
-#pragma unroll
-            for (int e = 0; e < L; ++e) {
-                if constexpr (FF) kahan_acc(shi[e], slo[e], acc[e]);
-                else s64[e] += widen(acc[e]);
-                acc[e] = 0.f;
-            }
+            if constexpr (FF) kahan_acc(shi, slo, acc);
+            else s64 += widen(acc);
+            acc = 0.f;
         }
     }
-#pragma unroll
-    for (int e = 0; e < L; ++e) {
-        if (e < RS) {
-            double sum;
-            if constexpr (FF) sum = pair_total(shi[e], slo[e], acc[e]);
-            else sum = s64[e] + widen(acc[e]);
-            double val = a.alpha == 1.0 ? sum : a.alpha * sum;
-            if (a.dtype == BSM_FP64) {
-                if (old >= 0) val = fma(a.beta, static_cast<const double *>(a.old_data)[old + e], val);
-                static_cast<double *>(a.out_data)[out_off + e] = val;
-            } else {
-                if (old >= 0) val = fma(a.beta, (double)static_cast<const float *>(a.old_data)[old + e], val);
-                static_cast<float *>(a.out_data)[out_off + e] = (float)val;
-            }
-        }
-    }
-}
-
-template <int PREC, bool FF, int R, int S>
-__device__ __forceinline__ void cs_lane_fixed(const NumericArgs &a, int64_t q) {
-    constexpr int NP = PrecTraits<PREC>::NP;
-    const float *__restrict__ X = a.x_plain;
-    const float *__restrict__ Y = a.y_plain;
-    const int64_t out_off = a.out_blk_off[q];
-    const int64_t p0 = a.seg_ptr[q], p1 = a.seg_ptr[q + 1];
-    const int64_t old = (a.beta != 0.0 && a.old_off) ? a.old_off[q] : -1;
-    const int F = a.flush_every > 0 ? a.flush_every : (a.flush_every < 0 ? -a.flush_every : 1);
-    float acc[R][S], shi[FF ? R : 1][FF ? S : 1], slo[FF ? R : 1][FF ? S : 1];
-    double s64[FF ? 1 : R][FF ? 1 : S];
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int c = 0; c < S; ++c) {
-            acc[r][c] = 0.f;
-            if constexpr (FF) {
-                shi[r][c] = 0.f;
-                slo[r][c] = 0.f;
-            } else {
-                s64[r][c] = 0.0;
-            }
-        }
-    int since = 0;
-    for (int64_t p = p0; p < p1; ++p) {
-        const int32_t ix = a.px[p], iy = a.py[p];
-        const float *xb = X + a.x_blk_off[ix] * NP;
-        const float *yb = Y + a.y_blk_off[iy] * NP;
-        const int32_t xrc = a.x_blk_rc[ix];
-        const int Tn = a.x_trans ? rc_rows(xrc) : rc_cols(xrc);
-        const int xs_r = a.x_trans ? 1 : Tn, xs_t = a.x_trans ? R : 1;
-        const int ys_t = a.y_trans ? 1 : S, ys_s = a.y_trans ? Tn : 1;
-        for (int t = 0; t < Tn; ++t) {
-            float xv[R][NP], yv[S][NP];
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-#pragma unroll
-                for (int pc = 0; pc < NP; ++pc) xv[r][pc] = __ldg(xb + (int64_t)(r * xs_r + t * xs_t) * NP + pc);
-#pragma unroll
-            for (int c = 0; c < S; ++c)
-#pragma unroll
-                for (int pc = 0; pc < NP; ++pc) yv[c][pc] = __ldg(yb + (int64_t)(t * ys_t + c * ys_s) * NP + pc);
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-#pragma unroll
-                for (int c = 0; c < S; ++c) {
-                    if constexpr (NP == 2) {
-                        acc[r][c] = fmaf(xv[r][1], yv[c][0], acc[r][c]);
-                        acc[r][c] = fmaf(xv[r][0], yv[c][1], acc[r][c]);
-                        acc[r][c] = fmaf(xv[r][0], yv[c][0], acc[r][c]);
-                    } else {
-                        acc[r][c] = fmaf(xv[r][2], yv[c][0], acc[r][c]);
-                        acc[r][c] = fmaf(xv[r][1], yv[c][1], acc[r][c]);
-                        acc[r][c] = fmaf(xv[r][0], yv[c][2], acc[r][c]);
-                        acc[r][c] = fmaf(xv[r][1], yv[c][0], acc[r][c]);
-                        acc[r][c] = fmaf(xv[r][0], yv[c][1], acc[r][c]);
-                        acc[r][c] = fmaf(xv[r][0], yv[c][0], acc[r][c]);
-                    }
-                }
-        }
-        if (++since == F) {
-            since = 0;
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-#pragma unroll
-                for (int c = 0; c < S; ++c) {
-                    if constexpr (FF) kahan_acc(shi[r][c], slo[r][c], acc[r][c]);
-                    else s64[r][c] += widen(acc[r][c]);
-                    acc[r][c] = 0.f;
-                }
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int c = 0; c < S; ++c) {
-            const int e = r * S + c;
-            double sum;
-            if constexpr (FF) sum = pair_total(shi[r][c], slo[r][c], acc[r][c]);
-            else sum = s64[r][c] + widen(acc[r][c]);
-            double val = a.alpha == 1.0 ? sum : a.alpha * sum;
-            if (a.dtype == BSM_FP64) {
-                if (old >= 0) val = fma(a.beta, static_cast<const double *>(a.old_data)[old + e], val);
-                static_cast<double *>(a.out_data)[out_off + e] = val;
-            } else {
-                if (old >= 0) val = fma(a.beta, (double)static_cast<const float *>(a.old_data)[old + e], val);
-                static_cast<float *>(a.out_data)[out_off + e] = (float)val;
-            }
-        }
-}
-
-template <int PREC, bool FF>
-__device__ __forceinline__ void cs_lane_dispatch(const NumericArgs &a, int64_t q) {
-    const int32_t orc = a.out_blk_rc[q];
-    switch ((rc_rows(orc) << 8) | rc_cols(orc)) {
-        case 0x101: cs_lane_fixed<PREC, FF, 1, 1>(a, q); break;
-        case 0x104: cs_lane_fixed<PREC, FF, 1, 4>(a, q); break;
-        case 0x401: cs_lane_fixed<PREC, FF, 4, 1>(a, q); break;
-        case 0x404: cs_lane_fixed<PREC, FF, 4, 4>(a, q); break;
-        case 0x202: cs_lane_fixed<PREC, FF, 2, 2>(a, q); break;
-        case 0x505: cs_lane_fixed<PREC, FF, 5, 5>(a, q); break;
-        default: cs_lane_item<PREC, FF>(a, q); break;
+    const double sum = FF ? pair_total(shi, slo, acc) : s64 + widen(acc);
+    double val = a.alpha == 1.0 ? sum : a.alpha * sum;
+    const int64_t out = a.out_blk_off[q] + e;
+    if (a.dtype == BSM_FP64) {
+        if (old >= 0) val = fma(a.beta, static_cast<const double *>(a.old_data)[old + e], val);
+        static_cast<double *>(a.out_data)[out] = val;
+    } else {
+        if (old >= 0) val = fma(a.beta, (double)static_cast<const float *>(a.old_data)[old + e], val);
+        static_cast<float *>(a.out_data)[out] = (float)val;
     }
 }
 
@@ -910,8 +776,9 @@ __global__ void __launch_bounds__(kThreadsNum) k_numeric_tc(NumericArgs a) {
 }
 
 // The last *n_lane_items items of the order: tiny blocks marked for the
-// CUDA-core variant, 32 per ticket (a kernel of their own, so that the
+// CUDA-core variant, kTinyItems per ticket (a kernel of their own, so that the
 // tensor-core instances do not carry its registers).
+constexpr int kTinyItems = 8;
 template <int PREC, bool FF>
 __global__ void __launch_bounds__(kThreadsNum) k_numeric_tc_lane(NumericArgs a) {
     const int lane = threadIdx.x & 31;
@@ -922,12 +789,21 @@ __global__ void __launch_bounds__(kThreadsNum) k_numeric_tc_lane(NumericArgs a) 
     while (true) {
         int64_t t = 0;
         if (lane == 0) t = (int64_t)atomicAdd(ctr, 1ull);
-        t = __shfl_sync(0xffffffffu, t, 0);
-        if (t * 32 >= n_lane) break;
-        const int64_t idx = lane0 + t * 32 + lane;
-        if (idx < a.n_items) {
-            const int64_t q = (int64_t)((uint32_t)a.item_order[idx] & 0x7fffffffu);
-            if (BSM_DBG_LANE_OK(a, q)) cs_lane_dispatch<PREC, FF>(a, q);
+        t = __shfl_sync(0xffffffffu, t, 0) * kTinyItems;
+        if (t >= n_lane) break;
+        int32_t q = -1;
+        int size = 0;
+        if (lane < kTinyItems && t + lane < n_lane) {
+            q = (int32_t)((uint32_t)a.item_order[lane0 + t + lane] & 0x7fffffffu);
+            const int32_t rc = a.out_blk_rc[q];
+            size = rc_rows(rc) * rc_cols(rc);
+        }
+        // lanes per block, by the ticket's largest
+        const int most = __reduce_max_sync(0xffffffffu, size), g = most <= 4 ? 4 : most <= 16 ? 16 : 32;
+        for (int i = lane / g; i - lane / g < kTinyItems; i += 32 / g) {
+            const int32_t qi = __shfl_sync(0xffffffffu, q, i);
+            const int e = lane % g;
+            if (e < __shfl_sync(0xffffffffu, size, i) && BSM_DBG_LANE_OK(a, qi)) cs_element<PREC, FF>(a, qi, e);
         }
     }
 }
@@ -1644,7 +1520,7 @@ cudaError_t launch_tc_ff(const NumericArgs &a, cudaStream_t s, int threads, int 
                     : launch_tc_pm<PREC, FF, 1>(b, s, threads, grid, pn);
     }
     if (e == cudaSuccess && a.n_lane_items) {
-        const int g = persistent_grid(k_numeric_tc_lane<PREC, FF>, a.n_items / 32 + 1, 0, kThreadsNum, a.ctas_per_sm);
+        const int g = persistent_grid(k_numeric_tc_lane<PREC, FF>, a.n_items / kTinyItems + 1, 0, kThreadsNum, a.ctas_per_sm);
         k_numeric_tc_lane<PREC, FF><<<g, kThreadsNum, 0, s>>>(a);
         count_launch(1);
         e = cudaGetLastError();
