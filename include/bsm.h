@@ -210,12 +210,12 @@ bsm_status bsm_get_launch_count(int64_t *count);
 /* Numeric variant per precision and output block shape (m rows, n columns),
  * for tiny blocks (m*n <= 16, 5 x 5, and on the FP64 and Ozaki paths 6 x 6;
  * other shapes always use variant 0):
- * 0 = one warp per output block (FP64_DMMA and FP32 data: lanes over its
- * elements; split and Ozaki paths: tensor-core MMA on packed fragments), 1 =
- * one lane per output block on CUDA cores (split paths: the same split pieces
- * multiplied with FP32 FMA, exact piece products; Ozaki path: plain FP64 FMA).
- * BSM_P_FP64 on FP64 data chooses the lanes of a block itself, whatever is set
- * here (the results are the same bits for any choice).  -1 restores the
+ * 0 = one warp per output block (FP64_DMMA: lanes over its elements; split and
+ * Ozaki paths: tensor-core MMA on packed fragments), 1 = CUDA cores, one lane
+ * per output block (FP64 FMA) or, on the split paths, per element (the same
+ * split pieces multiplied with FP32 FMA, exact piece products).  BSM_P_FP64 and
+ * FP32 data without a split choose the lanes of a block themselves, whatever is
+ * set here (the results are the same bits for any choice).  -1 restores the
  * library default (1 for m*n <= 16, 0 for 5 x 5 and 6 x 6);
  * bsm_get_variant returns the variant in effect.
  * Process-wide; the autotuner (paper_1708_03604_gb300/autotune.py) sets it

@@ -236,6 +236,7 @@ void free_pattern(bsm_mat *X) {
     dfree(X->t_ptr); X->t_ptr = nullptr;
     dfree(X->t_row); X->t_row = nullptr;
     dfree(X->t_blk); X->t_blk = nullptr;
+    dfree(X->t_bits); X->t_bits = nullptr;
     X->nnzb = 0;
     X->data_len = 0;
 }
@@ -586,7 +587,17 @@ bsm_status ensure_transpose(bsm_mat *X) {
     if (e == cudaSuccess) e = launch_gather_i32(n, tblk, rows, trow, g_stream);
     if (e == cudaSuccess) e = launch_histogram_u32(n, keys, X->nbc, counts, g_stream);
     if (e == cudaSuccess) e = launch_scan_i64(counts, tptr, X->nbc, stmp, g_stream);
+    // the columns' bitmaps, up to 256 MB
+    const int32_t words = (X->nbr + 31) / 32;
+    uint32_t *tbits = nullptr;
+    if (e == cudaSuccess && (int64_t)X->nbc * words <= (int64_t(1) << 26)) {
+        if ((st = sc.get(&tbits, (size_t)X->nbc * words))) return st;
+        e = cudaMemsetAsync(tbits, 0, sizeof(uint32_t) * (size_t)X->nbc * words, g_stream);
+        if (e == cudaSuccess) e = launch_col_bits(n, rows, X->col_idx, words, tbits, g_stream);
+    }
     if ((st = cuda_check(e, "transpose pattern"))) return st;
+    X->t_bits = tbits;
+    if (tbits) sc.release(tbits);
     X->t_ptr = tptr;
     X->t_row = trow;
     X->t_blk = tblk;
@@ -1388,6 +1399,12 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
 
     // ---- a2: symbolic count
     SymbolicArgs sa{};
+    if (use_filter) {
+        double *b_min;
+        if ((st = sc.get(&b_min, 1))) return st;
+        if ((st = cuda_check(launch_min_norm(B->nnzb, nB, b_min, g_stream), "smallest norm"))) return st;
+        sa.b_min = b_min;
+    }
     sa.nbr = nbr; sa.nbk = nbk; sa.nbc = nbc;
     sa.a_row_bs = A->row_bs; sa.a_col_bs = A->col_bs; sa.a_row_ptr = A->row_ptr; sa.a_col_idx = A->col_idx;
     sa.a_norm = nA;
@@ -1523,7 +1540,8 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
         FillOut f = fo;
         f.row0 = r0;
         f.prod_base = prod_base;
-        return by_cols ? launch_symbolic_fill_cols(sa, bitmaps, f, B->t_ptr, B->t_row, B->t_blk, g_stream, r1 - r0)
+        return by_cols ? launch_symbolic_fill_cols(sa, bitmaps, f, B->t_ptr, B->t_row, B->t_blk, B->t_bits, g_stream,
+                                                 r1 - r0)
                        : launch_symbolic_fill(sa, bitmaps, f, g_stream, r1 - r0);
     };
     if (!chunked) {  // a chunked multiply fills each row panel right before its numeric pass

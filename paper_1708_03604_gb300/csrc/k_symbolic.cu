@@ -377,15 +377,50 @@ __global__ void __launch_bounds__(kThreads) k_sym_fill(SymbolicArgs a, const uin
     }
 }
 
+// smallest norm (0 where one is NaN): every product of norms then exceeds a
+// threshold that the product of the two smallest exceeds, since rounding is
+// monotone
+__device__ __forceinline__ unsigned long long norm_key(double v) {
+    return v != v ? 0ull : (unsigned long long)__double_as_longlong(v);  // norms are not negative: ordered as integers
+}
+__global__ void __launch_bounds__(kThreads) k_min_norm(int64_t n, const double *norms, unsigned long long *out) {
+    __shared__ unsigned long long part;
+    if (threadIdx.x == 0) part = ~0ull;
+    __syncthreads();
+    unsigned long long m = ~0ull;
+    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n; b += (int64_t)gridDim.x * blockDim.x)
+        m = min(m, norm_key(norms[b]));
+    atomicMin(&part, m);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicMin(out, part);
+}
+
+__global__ void k_col_bits(int64_t n, const int32_t *rows, const int32_t *cols, int32_t words, uint32_t *bits) {
+    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n; b += (int64_t)gridDim.x * blockDim.x)
+        atomicOr(&bits[(int64_t)cols[b] * words + (rows[b] >> 5)], 1u << (rows[b] & 31));
+}
+
 // Fill through B's columns.  Same outputs as k_sym_fill, but every C block
-// (i, j) is built by walking B's column j (B transposed: ascending k) against
-// a shared-memory map k -> A block of row i, so its products come out in
-// ascending k already and are written contiguously (coalesced) instead of
-// scattered across the row's C blocks.
+// (i, j) is built from B's column j (B transposed: ascending k), so its
+// products come out in ascending k already and are written contiguously
+// (coalesced) instead of scattered across the row's C blocks.
+//
+// Where the filter can drop nothing of the row (no threshold, or the smallest
+// norms multiplied exceed it) the kept products of (i, j) are the common bits of
+// row i of A and column j of B: counting them reads a bit per inner block, and
+// the blocks' indices are ranks in the two bitmaps.  Elsewhere the column is
+// walked against a shared-memory map k -> A block of row i.  3,000 block rows of
+// 5/13/23 (2.5e8 products): the walk 8.6 ms, the bitmaps 2.5.
+constexpr int kFillWords = 32;                    // bitmap words a warp expands at a time
+struct FillWarp {
+    uint16_t list[kFillWords * 32];               // k of the products, relative to the first word
+    uint32_t bits[kFillWords], rank[kFillWords];  // column j's words, and its blocks before each
+};
 __global__ void __launch_bounds__(kThreads) k_sym_fill_cols(SymbolicArgs a, const uint32_t *bitmaps, FillOut o,
                                                             const int64_t *bt_ptr, const int32_t *bt_k,
-                                                            const int32_t *bt_b) {
+                                                            const int32_t *bt_b, const uint32_t *bt_bits) {
     extern __shared__ uint32_t smem[];
+    __shared__ unsigned long long a_min;
     __shared__ int32_t wtmp[32];
     if (a.status && *a.status != 0) return;
     const int nw = a.nwords;
@@ -440,8 +475,75 @@ __global__ void __launch_bounds__(kThreads) k_sym_fill_cols(SymbolicArgs a, cons
             o.old_off[crow + col_rank(bm, wpre, j)] = a.o_blk_off[c];
         }
     }
-    // pass 1: kept products per C block (one warp per C block)
     const unsigned lt = (1u << lane) - 1u;
+    // can the filter drop a product of this row?
+    bool all = bt_bits != nullptr;
+    if (all && a.use_filter) {
+        if (tid == 0) a_min = ~0ull;
+        __syncthreads();
+        unsigned long long key = ~0ull;
+        for (int64_t ai = a_beg + tid; ai < a_end; ai += blockDim.x) key = min(key, norm_key(a.a_norm[ai]));
+        atomicMin(&a_min, key);
+        __syncthreads();
+        all = a_beg == a_end || __dmul_rn(__longlong_as_double((long long)a_min), *a.b_min) > a.eps;
+        __syncthreads();
+    }
+    if (all) {
+        const int nk = (a.nbk + 31) >> 5;
+        uint32_t *abits = reinterpret_cast<uint32_t *>(amap);      // in place of the map
+        int32_t *apre = amap + nk;                                  // A's blocks before each word
+        FillWarp &fw = reinterpret_cast<FillWarp *>(amap + 2 * nk)[warp];
+        for (int w = tid; w < nk; w += blockDim.x) abits[w] = 0u;
+        __syncthreads();
+        for (int64_t ai = a_beg + tid; ai < a_end; ai += blockDim.x) {
+            const int32_t k = a.a_col_idx[ai];
+            atomicOr(&abits[k >> 5], 1u << (k & 31));
+        }
+        __syncthreads();
+        for (int w = tid; w < nk; w += blockDim.x) apre[w] = __popc(abits[w]);
+        __syncthreads();
+        block_exscan_array(apre, nk, wtmp);
+        for (int32_t r = warp; r < ccnt; r += nwarps) {
+            const uint32_t *col = bt_bits + (int64_t)o.c_col_idx[crow + r] * nk;
+            int32_t total = 0;
+            for (int w = lane; w < nk; w += 32) total += __popc(abits[w] & col[w]);
+            total = __reduce_add_sync(0xffffffffu, total);
+            if (lane == 0) cnt[r] = total;
+        }
+        __syncthreads();
+        block_exscan_array(cnt, ccnt, wtmp);
+        for (int32_t r = tid; r < ccnt; r += blockDim.x) o.cptr[crow + r] = prow + cnt[r];
+        for (int32_t r = warp; r < ccnt; r += nwarps) {
+            const int32_t j = o.c_col_idx[crow + r];
+            const uint32_t *col = bt_bits + (int64_t)j * nk;
+            const int32_t *blk = bt_b + bt_ptr[j];
+            int64_t cur = prow + cnt[r];
+            int32_t before = 0;  // column j's blocks before the words at hand
+            for (int w0 = 0; w0 < nk; w0 += kFillWords) {
+                const int w = w0 + lane;
+                const uint32_t cb = w < nk ? col[w] : 0u;
+                uint32_t both = w < nk ? cb & abits[w] : 0u;
+                const int32_t c_incl = warp_incl_scan(__popc(cb)), n = __popc(both), n_incl = warp_incl_scan(n);
+                fw.bits[lane] = cb;
+                fw.rank[lane] = (uint32_t)(before + c_incl - __popc(cb));
+                for (int32_t at = n_incl - n; both; both &= both - 1u) fw.list[at++] = (uint16_t)(32 * lane + __ffs(both) - 1);
+                __syncwarp();
+                const int32_t found = __shfl_sync(0xffffffffu, n_incl, 31);
+                for (int32_t q = lane; q < found; q += 32) {
+                    const int k = fw.list[q], kw = k >> 5;
+                    const uint32_t below = (1u << (k & 31)) - 1u;
+                    o.pa[cur + q] = (int32_t)a_beg + apre[w0 + kw] + __popc(abits[w0 + kw] & below);
+                    o.pb[cur + q] = blk[fw.rank[kw] + __popc(fw.bits[kw] & below)];
+                    o.pc[cur + q] = (int32_t)(crow + r);
+                }
+                cur += found;
+                before += __shfl_sync(0xffffffffu, c_incl, 31);
+                __syncwarp();
+            }
+        }
+        return;
+    }
+    // pass 1: kept products per C block (one warp per C block)
     for (int32_t r = warp; r < ccnt; r += nwarps) {
         const int32_t j = o.c_col_idx[crow + r];
         const int64_t cb = bt_ptr[j], ce = bt_ptr[j + 1];
@@ -841,12 +943,32 @@ int64_t symbolic_fill_smem_bytes(int32_t nwords, int32_t max_ccnt, int nchunk) {
 }
 
 int64_t symbolic_fill_cols_smem_bytes(int32_t nwords, int32_t max_ccnt, int32_t nbk) {
-    return (2 * (int64_t)nwords + (int64_t)max_ccnt + nbk + 1) * (int64_t)sizeof(int32_t);
+    // the map k -> A block, or row i's bitmap and ranks and the warps' lists
+    const int64_t map = std::max<int64_t>(nbk, 2 * (((int64_t)nbk + 31) / 32) +
+                                                   (int64_t)(kThreads / 32 * sizeof(FillWarp) / sizeof(int32_t)));
+    return (2 * (int64_t)nwords + (int64_t)max_ccnt + map + 1) * (int64_t)sizeof(int32_t);
+}
+
+cudaError_t launch_min_norm(int64_t n, const double *norms, double *out, cudaStream_t s) {
+    // 0x7f7f...: 1.4e306 (a bound that is too small only sends rows to the walk)
+    cudaError_t e = cudaMemsetAsync(out, 0x7f, sizeof(double), s);
+    if (e != cudaSuccess || n == 0) return e;
+    k_min_norm<<<std::min(grid_for(n), 152 * 4), kThreads, 0, s>>>(n, norms, reinterpret_cast<unsigned long long *>(out));
+    count_launch(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_col_bits(int64_t n, const int32_t *rows, const int32_t *cols, int32_t words, uint32_t *bits,
+                            cudaStream_t s) {
+    if (n == 0) return cudaSuccess;
+    k_col_bits<<<grid_for(n), kThreads, 0, s>>>(n, rows, cols, words, bits);
+    count_launch(1);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_symbolic_fill_cols(const SymbolicArgs &a, const uint32_t *bitmaps, const FillOut &o,
                                       const int64_t *bt_ptr, const int32_t *bt_k, const int32_t *bt_b,
-                                      cudaStream_t s, int32_t nrows) {
+                                      const uint32_t *bt_bits, cudaStream_t s, int32_t nrows) {
     if (nrows < 0) nrows = a.nbr - o.row0;
     if (nrows <= 0) return cudaSuccess;
     const int smem = (int)symbolic_fill_cols_smem_bytes(a.nwords, o.max_ccnt, a.nbk);
@@ -854,7 +976,7 @@ cudaError_t launch_symbolic_fill_cols(const SymbolicArgs &a, const uint32_t *bit
         cudaError_t e = cudaFuncSetAttribute(k_sym_fill_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
     }
-    k_sym_fill_cols<<<nrows, kThreads, smem, s>>>(a, bitmaps, o, bt_ptr, bt_k, bt_b);
+    k_sym_fill_cols<<<nrows, kThreads, smem, s>>>(a, bitmaps, o, bt_ptr, bt_k, bt_b, bt_bits);
     count_launch(1);
     return cudaGetLastError();
 }
