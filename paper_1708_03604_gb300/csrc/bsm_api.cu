@@ -472,13 +472,13 @@ bsm_status shape_order(Scratch &sc, int64_t n, const int32_t *blk_rc, const std:
     std::vector<int32_t> sidx(kMaxBlockDim + 1, 0), table((size_t)ns * ns);
     for (int32_t q = 0; q < ns; ++q) sidx[sizes[q]] = q;
     // with groups, the blocks a smaller kernel instance takes come after the
-    // others: split paths, one tile row (at most 16 rows); Ozaki path, one tile
-    // column (at most 8 columns)
+    // others: split paths, by height class; Ozaki path, one tile column (at most 8
+    // columns)
     const bool split = prec == BSM_P_TF32x3 || prec == BSM_P_BF16x3 || prec == BSM_P_BF16x6;
     const bool grouped = groups && (split || prec == BSM_P_OZAKI);
     auto group_of = [&](int32_t m, int32_t nn) -> int64_t {
         if (!grouped) return 0;
-        return (split ? m <= 16 : nn <= 8) ? 1 : 0;
+        return split ? split_group(m) : nn <= 8 ? 1 : 0;
     };
     std::vector<std::pair<int64_t, int32_t>> cls;
     for (int32_t r = 0; r < ns; ++r)
@@ -530,17 +530,17 @@ bsm_status shape_order(Scratch &sc, int64_t n, const int32_t *blk_rc, const std:
         e = launch_radix_sort_pairs(keys, iota, keys_alt, vals_alt, keys_sorted, out, n, bits, rtmp, g_stream);
     if ((st = cuda_check(e, "shape order"))) return st;
     if (grouped) {
-        // positions in the sorted order where group 1 and the lane items start
+        // positions in the sorted order where groups 1.. start
         const int64_t mult = use_tiles ? nrt * nct : (row_rank ? std::max(nbr, 1) : 1);
-        const int32_t ncls = (int32_t)cls.size();
-        int32_t q1 = 0;
-        while (q1 < ncls && group_of(sizes[cls[q1].second / ns], sizes[cls[q1].second % ns]) == 0) ++q1;
+        uint32_t thr[kSplitGroups - 1];
+        size_t q = 0;
+        for (int g = 0; g < kSplitGroups - 1; ++g) {
+            while (q < cls.size() && group_of(sizes[cls[q].second / ns], sizes[cls[q].second % ns]) <= g) ++q;
+            thr[g] = (uint32_t)(q * mult);
+        }
         int64_t *gb;
-        if ((st = sc.get(&gb, 2))) return st;
-        if ((st = cuda_check(launch_group_bounds(keys_sorted, n, (uint32_t)(q1 * mult), (uint32_t)(ncls * mult), gb,
-                                                 g_stream),
-                             "tile-row groups")))
-            return st;
+        if ((st = sc.get(&gb, kSplitGroups - 1))) return st;
+        if ((st = cuda_check(launch_group_bounds(keys_sorted, n, thr, gb, g_stream), "groups of blocks"))) return st;
         *groups = gb;
     }
     if (any_var) {
@@ -1686,7 +1686,7 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
         na.y_exp = olB.exps; na.y_line0 = olB.line0;
         na.status = no_sync ? C->status : nullptr;
         bsm_status sst;
-        if ((sst = sc.get(&na.work_counter, 4))) return sst;
+        if ((sst = sc.get(&na.work_counter, kWorkCounters))) return sst;
         if (no_sync) {
             order = C->item_order;
             n_marked = C->n_marked;
@@ -1709,6 +1709,7 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
                 return sst;
         }
         na.item_groups = groups;
+        for (int32_t m : A->h_row_bs) na.group_mask |= 1 << split_group(m);
         na.n_lane_items = n_marked;
         if (needs_plain(kprec) && uses_cores && !plain_x) {  // unpacked pieces for the CUDA-core split variant
             const int np = split_pieces(rprec);
@@ -1963,15 +1964,22 @@ bsm_status bsm_multiply_backward(double alpha, bsm_t C, const void *dC_data, bsm
         na.y_pack = pkY.words; na.y_pack_off = pkY.off;
         na.x_exp = olX.exps; na.x_line0 = olX.line0;
         na.y_exp = olY.exps; na.y_line0 = olY.line0;
-        if ((st = sc.get(&na.work_counter, 4))) return st;
+        if ((st = sc.get(&na.work_counter, kWorkCounters))) return st;
         int32_t *item_order = nullptr;
         int64_t *n_marked = nullptr;
         bool uses_cores = false;
+        // one kernel instance per height class where it adds in the same order
+        // (more block products per sum run two accumulators in some of them)
+        const bool want_groups = is_tc(kprec) && kprec != BSM_P_OZAKI && std::abs(opts.flush_every) <= 1 &&
+                                 tune_of(opts.prec)[BSM_TUNE_PASS_MT] <= 0;
+        int64_t *groups = nullptr;
         if ((st = shape_order(sc, OUT->nnzb, OUT->blk_rc, OUT->h_row_bs, OUT->h_col_bs, &item_order, nullptr, nullptr,
                               kprec == BSM_P_FP64 || (kprec == BSM_P_FP64_DMMA && C->dtype != BSM_FP64) ? -1 : opts.prec,
-                              &uses_cores, &n_marked)))
+                              &uses_cores, &n_marked, nullptr, nullptr, 0, 0, want_groups ? &groups : nullptr)))
             return st;
         na.n_lane_items = n_marked;
+        na.item_groups = groups;
+        for (int32_t m : OUT->h_row_bs) na.group_mask |= 1 << split_group(m);
         if (needs_plain(kprec) && uses_cores && nprod > 0) {
             const int np = split_pieces(opts.prec);
             float *xp = nullptr, *yp = nullptr;

@@ -91,7 +91,7 @@ struct bsm_mat {
     } plan;
     int32_t *item_order = nullptr;      // numeric processing order of the last eager multiply
     int64_t *n_marked = nullptr;        // device count of its second-variant items (or null)
-    int64_t *item_groups = nullptr;     // device bounds of its tile-row groups (or null)
+    int64_t *item_groups = nullptr;     // device bounds of its groups of blocks (or null)
     // rank of every block row in a breadth-first order through shared block
     // columns (built on demand, dropped with the pattern); schedules numeric work
     int32_t *row_rank = nullptr;        // [nbr]
@@ -253,6 +253,13 @@ cudaError_t launch_class_keys(int64_t n, const int32_t *blk_rc, const int32_t *s
                               const int32_t *blk_col, const int32_t *col_rank, int32_t tile, int32_t nct,
                               uint32_t *keys, int32_t *iota, cudaStream_t s);
 
+// Height classes of the split paths' output blocks, in the order they run: more
+// than 24 rows, 17 to 24, 9 to 16, at most 8 (the second and the last end in half
+// a tile row)
+constexpr int kSplitGroups = 4;
+inline int split_group(int rows) { return rows > 24 ? 0 : rows > 16 ? 1 : rows > 8 ? 2 : 3; }
+constexpr int kWorkCounters = kSplitGroups + 1;  // tickets of the groups and of the lane items
+
 // ---------------------------------------------------------------- numeric
 struct NumericArgs {
     int64_t n_items;
@@ -283,13 +290,14 @@ struct NumericArgs {
                                 // bit 31 marks the second variant of the item's shape
     const int64_t *n_lane_items;  // nullable (CUDA-core FP64 path): the last *n_lane_items items of
                                   // item_order are tiny blocks computed one per lane
-    // nullable (split paths): item_order positions [0] end of the blocks of two
-    // tile rows and more, [1] end of the blocks of one tile row (start of the
-    // lane items); each group runs in its own kernel instance
+    // nullable: item_order positions where the next group of blocks starts, one
+    // kernel instance each.  Split paths: kSplitGroups height classes (split_group);
+    // Ozaki path: two groups, the second of blocks of one tile column
     const int64_t *item_groups;
+    int32_t group_mask;         // the groups that the output's block sizes can fill
     int32_t group;              // set by the launcher: the group one launch covers
     const int32_t *status;      // nullable: the kernel does nothing when *status != 0
-    unsigned long long *work_counter;  // 4 x 8 bytes of device memory, zeroed by the launcher
+    unsigned long long *work_counter;  // kWorkCounters x 8 bytes of device memory, zeroed by the launcher
     // Ozaki path: biased FP64 exponent field of the largest |x| of every global
     // line (logical rows of X, logical columns of Y) and the first line of every block
     const int32_t *x_exp, *x_line0, *y_exp, *y_line0;
@@ -322,10 +330,16 @@ cudaError_t launch_numeric_group(const NumericArgs &a, int build, cudaStream_t s
 uint32_t group_debug_bits(cudaStream_t s);
 // FP32 data on the CUDA cores (k_tile.cu)
 cudaError_t launch_numeric_tile(const NumericArgs &a, cudaStream_t s, int *grid);
+cudaError_t launch_split_tf32x3(const NumericArgs &a, cudaStream_t s, int threads, int *grid);
+cudaError_t launch_split_bf16x3(const NumericArgs &a, cudaStream_t s, int threads, int *grid);
+cudaError_t launch_split_bf16x6(const NumericArgs &a, cudaStream_t s, int threads, int *grid);
+uint32_t split_tf32x3_debug_bits(cudaStream_t s);
+uint32_t split_bf16x3_debug_bits(cudaStream_t s);
+uint32_t split_bf16x6_debug_bits(cudaStream_t s);
 uint32_t tile_debug_bits(cudaStream_t s);
 int num_sms();
 // out[g] = number of keys below thr[g] in the ascending keys[0..n) (g < 2)
-cudaError_t launch_group_bounds(const uint32_t *keys, int64_t n, uint32_t thr0, uint32_t thr1, int64_t *out,
+cudaError_t launch_group_bounds(const uint32_t *keys, int64_t n, const uint32_t (&thr)[kSplitGroups - 1], int64_t *out,
                                 cudaStream_t s);
 
 // Ozaki path: line0[b] = first global line of block b, lines being the stored

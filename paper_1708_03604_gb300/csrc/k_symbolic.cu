@@ -858,11 +858,12 @@ __global__ void k_class_keys(int64_t n, const int32_t *blk_rc, const int32_t *si
     }
 }
 
-// lower bounds of two thresholds in sorted keys (one thread each)
-__global__ void k_group_bounds(const uint32_t *keys, int64_t n, uint32_t thr0, uint32_t thr1, int64_t *out) {
+// lower bounds of thresholds in sorted keys (one thread each)
+struct GroupThr { uint32_t v[kSplitGroups - 1]; };
+__global__ void k_group_bounds(const uint32_t *keys, int64_t n, GroupThr t, int64_t *out) {
     const int g = threadIdx.x;
-    if (g >= 2) return;
-    const uint32_t thr = g == 0 ? thr0 : thr1;
+    if (g >= kSplitGroups - 1) return;
+    const uint32_t thr = t.v[g];
     int64_t lo = 0, hi = n;
     while (lo < hi) {
         const int64_t mid = (lo + hi) >> 1;
@@ -882,9 +883,11 @@ inline int grid_for(int64_t n, int threads = kThreads) {
 }  // namespace
 
 // =================================================================== launchers
-cudaError_t launch_group_bounds(const uint32_t *keys, int64_t n, uint32_t thr0, uint32_t thr1, int64_t *out,
-                                cudaStream_t s) {
-    k_group_bounds<<<1, 32, 0, s>>>(keys, n, thr0, thr1, out);
+cudaError_t launch_group_bounds(const uint32_t *keys, int64_t n, const uint32_t (&thr)[kSplitGroups - 1],
+                                int64_t *out, cudaStream_t s) {
+    GroupThr t;
+    for (int g = 0; g < kSplitGroups - 1; ++g) t.v[g] = thr[g];
+    k_group_bounds<<<1, 32, 0, s>>>(keys, n, t, out);
     count_launch(1);
     return cudaGetLastError();
 }

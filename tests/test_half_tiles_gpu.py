@@ -1,0 +1,50 @@
+"""The split paths' half tiles (GPU): where at most 8 rows of an output block
+fall into its last tile row, the packs, copies and sums of the empty half fall
+away.  Heights on both sides of every edge.  Against the oracle the bound of the
+path (1e-6, the two-piece BF16 split 1e-4); kernels for blocks of one height
+class and the one for any height run every element through the same chain of
+sums, so they must agree bit for bit (one block product a sum)."""
+import numpy as np
+import pytest
+
+from paper_1708_03604_gb300 import inputs as I
+from tests.helpers import random_bcsr, rel_fro
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"tf32x3": 1e-6, "bf16x6": 1e-6, "bf16x3": 1e-4}
+
+
+@pytest.fixture(scope="module")
+def bsm():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1708_03604_gb300 import bsm as B
+    B.lib()
+    return B
+
+
+@pytest.mark.parametrize("heights", [(5, 8, 9), (16, 17, 24), (23, 25, 32), (33, 40, 41), (48, 56, 7)], ids=str)
+@pytest.mark.parametrize("prec", sorted(TOL))
+def test_heights(bsm, oracle, prec, heights):
+    from paper_1708_03604_gb300 import autotune
+    rows = I.mixed_sizes(40, heights, [1 / 3] * 3, seed=3)
+    mid = I.mixed_sizes(40, (3, 8, 17), [1 / 3] * 3, seed=4)
+    cols = I.mixed_sizes(40, (6, 13, 24), [1 / 3] * 3, seed=5)
+    Ah, Bh = random_bcsr(rows, mid, 0.3, seed=6), random_bcsr(mid, cols, 0.3, seed=7)
+    C0 = random_bcsr(rows, cols, 0.4, seed=8)
+    A, B = bsm.Matrix.from_host(Ah), bsm.Matrix.from_host(Bh)
+    ref = oracle.multiply(1.5, Ah, Bh, 0.5, C0)
+    for flush in (0, 1, -3, 4):
+        got = {}
+        try:
+            for pm in (-1, 2, 1):
+                bsm.bsm_set_tuning(prec, "pass_mt", pm)
+                got[pm] = bsm.multiply(1.5, A, B, 0.5, bsm.Matrix.from_host(C0), prec=prec, flush_every=flush).data_host()
+        finally:
+            autotune.reset(prec)
+        for pm, c in got.items():
+            assert rel_fro(c, ref.C.data) <= TOL[prec], (flush, pm)
+            if flush in (0, 1):
+                np.testing.assert_array_equal(c, got[-1])
