@@ -257,6 +257,16 @@ bool is_tc(int prec) {
     return prec == BSM_P_TF32x3 || prec == BSM_P_BF16x3 || prec == BSM_P_BF16x6 || prec == BSM_P_OZAKI;
 }
 // split paths whose lane variant multiplies unpacked FP32 pieces
+// the kernel instances that output blocks of these heights and products of these
+// inner sizes need
+void tile_masks(const std::vector<int32_t> &rows, const std::vector<int32_t> &inner, NumericArgs &na) {
+    for (int32_t k : inner) na.half_mask |= half_rows(k) ? kHalfInner : 0;
+    for (int32_t m : rows) {
+        na.group_mask |= 1 << split_group(m);
+        na.half_mask |= (half_rows(m) ? kHalfRows : 0) | (m > 8 ? kWholeRows : 0);
+    }
+}
+
 bool needs_plain(int prec) { return is_tc(prec) && prec != BSM_P_OZAKI; }
 
 // first global row / column of every block row / column, on the device
@@ -1709,7 +1719,7 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
                 return sst;
         }
         na.item_groups = groups;
-        for (int32_t m : A->h_row_bs) na.group_mask |= 1 << split_group(m);
+        tile_masks(A->h_row_bs, A->h_col_bs, na);
         na.n_lane_items = n_marked;
         if (needs_plain(kprec) && uses_cores && !plain_x) {  // unpacked pieces for the CUDA-core split variant
             const int np = split_pieces(rprec);
@@ -1979,7 +1989,7 @@ bsm_status bsm_multiply_backward(double alpha, bsm_t C, const void *dC_data, bsm
             return st;
         na.n_lane_items = n_marked;
         na.item_groups = groups;
-        for (int32_t m : OUT->h_row_bs) na.group_mask |= 1 << split_group(m);
+        tile_masks(OUT->h_row_bs, side == 0 ? B->h_col_bs : A->h_row_bs, na);
         if (needs_plain(kprec) && uses_cores && nprod > 0) {
             const int np = split_pieces(opts.prec);
             float *xp = nullptr, *yp = nullptr;

@@ -257,6 +257,11 @@ cudaError_t launch_class_keys(int64_t n, const int32_t *blk_rc, const int32_t *s
 // than 24 rows, 17 to 24, 9 to 16, at most 8 (the second and the last end in half
 // a tile row)
 constexpr int kSplitGroups = 4;
+// Ozaki path: whether at most 8 rows (or terms of k) fall into the last tile of 16
+__host__ __device__ constexpr bool half_rows(int rows) { return ((rows - 1) & 15) < 8; }
+// some output block ends in half a tile row; some has a whole one; some product
+// ends in half a k-step
+constexpr int kHalfRows = 1, kWholeRows = 2, kHalfInner = 4;
 inline int split_group(int rows) { return rows > 24 ? 0 : rows > 16 ? 1 : rows > 8 ? 2 : 3; }
 constexpr int kWorkCounters = kSplitGroups + 1;  // tickets of the groups and of the lane items
 
@@ -295,6 +300,7 @@ struct NumericArgs {
     // Ozaki path: two groups, the second of blocks of one tile column
     const int64_t *item_groups;
     int32_t group_mask;         // the groups that the output's block sizes can fill
+    int32_t half_mask;          // Ozaki path: kHalfRows | kWholeRows | kHalfInner
     int32_t group;              // set by the launcher: the group one launch covers
     const int32_t *status;      // nullable: the kernel does nothing when *status != 0
     unsigned long long *work_counter;  // kWorkCounters x 8 bytes of device memory, zeroed by the launcher
