@@ -635,7 +635,7 @@ def run_headline(args, name, world, rank, local_rank):
     shapes, scounts = Cm[0].stack_shapes()
     roofline = leg_roofline("fp64", flop, None, num_ms, peaks, tpk)
     traffic = traffic_from_profile(name) if world == 1 else None
-    roofline.update(kernel=("k_numeric_cc<double> (FP64 FMA, one warp per C block; stream of the multiply, "
+    roofline.update(kernel=("k_numeric_group (FP64 FMA, one warp per C block of this size; stream of the multiply, "
                             "CUDA events of the library around the launch)"),
                     traffic=traffic,
                     traffic_note=("dram__bytes_read.sum + dram__bytes_write.sum of one launch at 2000 block rows, "

@@ -10,7 +10,7 @@ recorded by the library around the launch) on the caller's operands:
   fragments) or, for blocks of at most 16 elements and 5 x 5 ones (FP64 and
   Ozaki also 6 x 6), one lane per block on the CUDA cores;
 * the FP64 FMA kernel build (how many output elements a lane holds per pass:
-  up to 9 or up to 24) -- BSM_P_FP64;
+  up to 13 or up to 24) -- BSM_P_FP64;
 * warps per CTA (4 or 2) of the persistent mma.sync kernels;
 * persistent CTAs per SM;
 * the fragment-tile pass shape (tiles along rows and columns that one pass
@@ -55,7 +55,7 @@ SEARCH = {
     "ozaki": [("cta_warps", [4, 2]), ("pass_nt", [3, 2, 1]), ("ctas_per_sm", [0, 1, 2, 3]), TILES],
 }
 for _p in SPLIT:
-    # pass_mt -1: blocks of one tile row in a 1-row kernel instance, the rest in a 2-row one
+    # pass_mt -1: a kernel instance per height class of the blocks
     SEARCH[_p] = [("cta_warps", [4, 2]), ("pass_mt", [-1, 2, 1]), ("pass_nt", [3, 2, 1]),
                   ("ctas_per_sm", [0, 1, 2, 3, 4]), TILES]
 # TF32x3 may also run on the tcgen05 row-panel engine where it applies

@@ -427,8 +427,8 @@ __host__ __device__ constexpr int oz_ring_words_per_warp() { return kOzStages * 
 //   both  chunk c = v0 of p = 4c, p + 1, p + 2, p + 3 against Y {q, q-2}: level
 //       p + q from p and p + 2 below, level p + q + 1 from p + 1 and p + 3 above
 // With HK the Y slices are words, 4c..4c+3 in chunk c.  21 MMAs a tile and k-step
-// become 12, 12 and 8.  (Zeros in the empty half, with or without m16n8k8, cost
-// more than they saved: each MMA's registers had to be put together by moves.)
+// become 12, 12 and 8.  (The same packs with zeros in the empty half were slower
+// than whole tiles: 2,000 banded rows of 23 62.5 ms, 57.3 with m16n8k8, against 55.0.)
 
 // The MMAs of one k-step from its ring stage (w: this lane's words).  acc[l]: level
 // l; with HM level l in rows 0..7, level l + 1 in rows 8..15 (of acc[5] not used).
