@@ -143,6 +143,15 @@ inline bsm_status dalloc_t(T **p, size_t n) {
     return dalloc(reinterpret_cast<void **>(p), n * sizeof(T) + (n == 0 ? 16 : 0));
 }
 
+// Dynamic shared memory for a launch of `kernel`.  Its static and dynamic arrays
+// together are held to 48 KB unless it opts in to more; the static arrays of the
+// kernels that size the dynamic part from their operands are below 2 KB.
+template <typename K>
+inline cudaError_t allow_dynamic_smem(K *kernel, size_t bytes) {
+    if (bytes <= 46 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 // ---------------------------------------------------------------- launchers
 // (all asynchronous on `s`; they return cudaGetLastError())
 cudaError_t launch_blk_rc(const bsm_mat *X, int32_t *out_rc, cudaStream_t s);

@@ -189,10 +189,8 @@ extern "C" bsm_status bsm_count_products_static(bsm_t A, bsm_t B, double filter_
     sa.eps = filter_eps;
     sa.use_filter = use_filter ? 1 : 0;
     sa.nwords = nwords;
-    if (smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(k_sym_count_static, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute");
-    }
+    if ((e = allow_dynamic_smem(k_sym_count_static, (size_t)smem)) != cudaSuccess)
+        return cuda_check(e, "cudaFuncSetAttribute");
     k_sym_count_static<<<A->nbr, kThreads, smem, s>>>(sa, prod_cnt, cblk_cnt,
                                                       reinterpret_cast<unsigned long long *>(totals));
     count_launch(1);

@@ -935,10 +935,7 @@ cudaError_t launch_panel_tiles_count(int32_t nbr, const int32_t *ord_r, const in
     const int32_t ngr = (nbr + kRB - 1) / kRB;
     if (ngr == 0) return cudaSuccess;
     const size_t smem = panel_tile_smem(ngc) / 2;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_panel_tile_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_dynamic_smem(k_panel_tile_count, smem)) return e;
     k_panel_tile_count<<<ngr, 128, smem, s>>>(nbr, ord_r, pos_c, c_row_ptr, c_col, ngc, tile_cnt);
     count_launch(1);
     return cudaGetLastError();
@@ -951,10 +948,7 @@ cudaError_t launch_panel_tiles_fill(int32_t nbr, const int32_t *ord_r, const int
     const int32_t ngr = (nbr + kRB - 1) / kRB;
     if (ngr == 0) return cudaSuccess;
     const size_t smem = panel_tile_smem(ngc);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_panel_tile_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_dynamic_smem(k_panel_tile_fill, smem)) return e;
     k_panel_tile_fill<<<ngr, 128, smem, s>>>(nbr, ord_r, pos_c, c_row_ptr, c_col, ngc, tile_ptr, tile_g, tile_h,
                                              cblk);
     count_launch(1);
@@ -975,6 +969,7 @@ cudaError_t launch_panel_steps(const PanelArgs &a, int fill, int64_t *step_cnt, 
     const int nw = (a.nbk + 31) >> 5;
     const size_t smem = (size_t)(2 * kBmLists + 2) * nw * sizeof(uint32_t);
     if (nw > 0 && smem <= 48 * 1024 && a.n_tiles < (int64_t(1) << 31)) {
+        if (const cudaError_t e = allow_dynamic_smem(k_panel_steps_bm, smem)) return e;
         k_panel_steps_bm<<<(unsigned)a.n_tiles, 128, smem, s>>>(a, fill, step_cnt);
     } else {  // the bitmaps do not fit: the warp-per-tile merge
         k_panel_steps<<<(unsigned)((a.n_tiles * 32 + 255) / 256), 256, 0, s>>>(a, fill, step_cnt);

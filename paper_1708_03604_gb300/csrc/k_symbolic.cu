@@ -931,11 +931,7 @@ cudaError_t launch_symbolic_count(const SymbolicArgs &a, int64_t *prod_cnt, int6
                                   cudaStream_t s) {
     if (a.nbr == 0) return cudaSuccess;
     const size_t smem = (size_t)a.nwords * sizeof(uint32_t);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_sym_count, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_dynamic_smem(k_sym_count, smem)) return e;
     k_sym_count<<<a.nbr, kThreads, smem, s>>>(a, prod_cnt, ccol_cnt, celem_cnt, bitmaps, totals);
     count_launch(1);
     return cudaGetLastError();
@@ -975,10 +971,7 @@ cudaError_t launch_symbolic_fill_cols(const SymbolicArgs &a, const uint32_t *bit
     if (nrows < 0) nrows = a.nbr - o.row0;
     if (nrows <= 0) return cudaSuccess;
     const int smem = (int)symbolic_fill_cols_smem_bytes(a.nwords, o.max_ccnt, a.nbk);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_sym_fill_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_dynamic_smem(k_sym_fill_cols, smem)) return e;
     k_sym_fill_cols<<<nrows, kThreads, smem, s>>>(a, bitmaps, o, bt_ptr, bt_k, bt_b, bt_bits);
     count_launch(1);
     return cudaGetLastError();
@@ -996,10 +989,7 @@ cudaError_t launch_symbolic_fill(const SymbolicArgs &a, const uint32_t *bitmaps,
     if (nrows < 0) nrows = a.nbr - o.row0;
     if (nrows <= 0) return cudaSuccess;
     const int smem = (int)symbolic_fill_smem_bytes(a.nwords, o.max_ccnt, o.nchunk);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_sym_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_dynamic_smem(k_sym_fill, smem)) return e;
     k_sym_fill<<<nrows, kThreads, smem, s>>>(a, bitmaps, o);
     count_launch(1);
     return cudaGetLastError();
