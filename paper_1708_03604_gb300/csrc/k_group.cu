@@ -39,6 +39,10 @@ constexpr uint32_t kQNarrow = kQSmall | q_bit(5) | q_bit(6) | q_bit(7) | q_bit(8
 constexpr uint32_t kQWide = kQNarrow | q_bit(15) | q_bit(17) | q_bit(19) | q_bit(21) | q_bit(24);
 // Q of the layouts whose lanes keep one row or one column
 constexpr uint32_t kQShared = kQNarrow;
+// whether Q = q is compiled into a build; any q (a shift by 32 is undefined)
+__host__ __device__ constexpr bool has_q(uint32_t mask, int q) { return q < 32 && ((mask >> q) & 1u); }
+static_assert(has_q(kQWide, 24) && !has_q(kQWide, 31) && !has_q(kQWide, 32));
+static_assert(has_q(kQSmall, 1) && has_q(kQNarrow, 1) && has_q(kQWide, 1));
 
 template <int BUILD>
 __host__ __device__ constexpr uint32_t q_mask() {
@@ -86,7 +90,7 @@ __device__ GroupPlan group_plan(int m, int n, bool spread, int lane) {
             best_g = g;
         }
     };
-    if ((MASK >> (lane + 1)) & 1u) {
+    if (has_q(MASK, lane + 1)) {
         const int q = lane + 1, rows = min(min(m, (31 + n) / n + 1), blk_lines), cols = (min(32, n) * 8 >> 7) + 1;
         rate(kFlat, q, 32, 1, (rs + 32 * q - 1) / (32 * q), q * (rows + cols));
     }
@@ -103,8 +107,11 @@ __device__ GroupPlan group_plan(int m, int n, bool spread, int lane) {
     }
     const uint32_t top = __reduce_min_sync(0xffffffffu, best);
     const int win = __ffs(__ballot_sync(0xffffffffu, best == top)) - 1;
-    return GroupPlan{__shfl_sync(0xffffffffu, best_mode, win), __shfl_sync(0xffffffffu, best_q, win),
-                     __shfl_sync(0xffffffffu, best_g, win)};
+    const GroupPlan pl{__shfl_sync(0xffffffffu, best_mode, win), __shfl_sync(0xffffffffu, best_q, win),
+                       __shfl_sync(0xffffffffu, best_g, win)};
+    // only layouts that are compiled are rated; a block without one would never be
+    // taken from the window, so it would go to one that takes every shape
+    return has_q(pl.mode == kFlat ? MASK : MASK & kQShared, pl.q) ? pl : GroupPlan{kFlat, 1, 32};
 }
 
 // Blocks of shape m x n from `run`, until the next one has another shape or
@@ -351,7 +358,7 @@ k_numeric_group(NumericArgs a) {
         switch (pl.mode * 32 + pl.q) {
 #define BSM_Q_MODE(Q, MODE, MASK_)                                                   \
     case MODE * 32 + Q:                                                              \
-        if constexpr (((MASK_) >> Q) & 1u) group_run<Q, MODE>(a, run, lane, m, n, pl.g); \
+        if constexpr (has_q(MASK_, Q)) group_run<Q, MODE>(a, run, lane, m, n, pl.g); \
         break;
 #define BSM_Q(Q) BSM_Q_MODE(Q, kFlat, MASK) BSM_Q_MODE(Q, kRow, MASK &kQShared) BSM_Q_MODE(Q, kCol, MASK &kQShared)
             BSM_Q(1) BSM_Q(2) BSM_Q(3) BSM_Q(4) BSM_Q(5) BSM_Q(6) BSM_Q(7) BSM_Q(8)

@@ -302,7 +302,10 @@ __global__ void __launch_bounds__(kGroupThreads, ROWS == 4 ? 5 : 4) k_numeric_ti
         const int32_t rc = run.w->shape[run.cur];
         const int m = rc_rows(rc), n = rc_cols(rc);
         const TilePlan pl = tile_plan<ROWS>(m, n, spread, a, lane);
+        // one element per lane in as many passes as it takes, the default, takes every
+        // shape: whatever the plan, the run ends
         switch (pl.tr * 8 + pl.tc) {
+            default:
 #define BSM_TILE(TR, TC) \
     case TR * 8 + TC:                                                             \
         if constexpr (TR <= ROWS) tile_run<TR, TC>(a, run, lane, m, n, pl.lr, pl.lc); \
