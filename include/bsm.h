@@ -103,7 +103,10 @@ typedef struct {
                               compensated FP32 pair (Kahan) refreshed every -F
                               products, converted to FP64 at the end; 0: as -1.
                               Range [-1024, 1024].  BSM_P_OZAKI ignores it (its
-                              flushes follow from the exact-sum bound).            */
+                              flushes follow from the exact-sum bound).  FP32 data
+                              on the CUDA cores: F > 0 adds the FP32 sum of F
+                              products in FP64, else every product (see also
+                              bsm_set_variant)                                     */
     int32_t no_sync;       /* 1: no host synchronisation (CUDA-graph capturable); see
                               bsm_multiply and bsm_add                               */
     int32_t reserved[3];   /* must be zero                                          */
@@ -215,9 +218,10 @@ bsm_status bsm_get_launch_count(int64_t *count);
  * per output block (FP64 FMA) or, on the split paths, per element (the same
  * split pieces multiplied with FP32 FMA, exact piece products).  BSM_P_FP64 and
  * FP32 data without a split choose the lanes of a block themselves, whatever is
- * set here (the results are the same bits for any choice).  -1 restores the
- * library default (1 for m*n <= 16, 0 for 5 x 5 and 6 x 6);
- * bsm_get_variant returns the variant in effect.
+ * set here; FP64 results are the same bits for either, and FP32 data adds every
+ * block product in FP64 with 1 and flush_every of them together with 0.  -1
+ * restores the library default (1 for m*n <= 16, 0 for 5 x 5 and 6 x 6);
+ * bsm_get_variant returns the variant set, or the default.
  * Process-wide; the autotuner (paper_1708_03604_gb300/autotune.py) sets it
  * from measurements.  Applies to multiplies issued afterwards (a no-sync
  * multiply keeps the choice of its eager call).  BSM_P_TF32x3_PANEL has no

@@ -54,6 +54,15 @@ int variant_of(int prec, int m, int n) {
     if (v >= 0) return v;
     return m * n <= 16 ? 1 : 0;
 }
+// the shapes of variant 1, which adds every block product of FP32 data in FP64
+EachProduct each_product_of(int prec) {
+    EachProduct each;
+    for (int m = 1; m <= 16; ++m)
+        for (int n = 1; n <= 16; ++n)
+            if (variant_of(prec, m, n) == 1) each.cols[m - 1] |= 1u << (n - 1);
+    return each;
+}
+
 // true when every output block shape (a row size of `rows` by a column size
 // of `cols`) runs the lane-per-block variant for `prec`
 bool all_lane(int prec, const std::vector<int32_t> &rows, const std::vector<int32_t> &cols) {
@@ -1690,6 +1699,7 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
         na.flush_every = opts.flush_every;
         na.max_out_rows = A->max_bs_row; na.max_out_cols = B->max_bs_col;
         na.mixed_k = mixed_sizes(A->h_col_bs);
+        if (A->dtype != BSM_FP64) na.each_product = no_sync ? pl.each_product : each_product_of(rprec);
         na.x_pack = pkA.words; na.x_pack_off = pkA.off;
         na.y_pack = pkB.words; na.y_pack_off = pkB.off;
         na.x_exp = olA.exps; na.x_line0 = olA.line0;
@@ -1820,6 +1830,7 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
         P.kind = 1; P.A = A; P.B = B; P.A_nnzb = A->nnzb; P.B_nnzb = B->nnzb; P.eps = filter_eps;
         P.prec = opts.prec; P.kprec = kprec; P.nprod = nprod; P.nnzb = nnzbC; P.len = lenC; P.max_ccnt = max_ccnt;
         P.uses_cores = uses_cores;
+        if (A->dtype != BSM_FP64) P.each_product = each_product_of(rprec);
         P.nfilt = nfilt; P.mnk = mnk; P.nchunk = nchunk; P.packA = packA_words; P.packB = packB_words;
     }
 
@@ -1969,6 +1980,7 @@ bsm_status bsm_multiply_backward(double alpha, bsm_t C, const void *dC_data, bsm
         na.prec = kprec;
         na.max_out_rows = OUT->max_bs_row; na.max_out_cols = OUT->max_bs_col;
         na.mixed_k = mixed_sizes(side == 0 ? B->h_col_bs : A->h_row_bs);
+        if (C->dtype != BSM_FP64) na.each_product = each_product_of(opts.prec);
         na.flush_every = opts.flush_every;
         na.x_pack = pkX.words; na.x_pack_off = pkX.off;
         na.y_pack = pkY.words; na.y_pack_off = pkY.off;

@@ -28,6 +28,13 @@ __host__ __device__ inline int rc_cols(int32_t rc) { return (int)(rc & 0xffff); 
 // Status bits written by kernels into a per-call device word.
 enum : int32_t { DEV_OK = 0, DEV_ERR_CAPACITY = 1, DEV_ERR_RANGE = 2 };
 
+// FP32 data without a split: the output block shapes (up to 16 x 16) whose block
+// products are added one by one in FP64, flush_every together elsewhere
+struct EachProduct {
+    uint16_t cols[16] = {};  // bit n - 1 of entry m - 1
+    __host__ __device__ bool has(int m, int n) const { return m <= 16 && n <= 16 && (cols[m - 1] >> (n - 1) & 1); }
+};
+
 // One stored operand view for the numeric kernels: element (r, t) of the
 // logical R x T block is data[off + (trans ? t*R + r : r*T + t)], where the
 // stored block is R x T (trans = 0) or T x R (trans = 1).
@@ -87,6 +94,7 @@ struct bsm_mat {
         int32_t nchunk = 1;
         int64_t packA = 0, packB = 0;
         bool uses_cores = false;  // some items run the CUDA-core split variant
+        bsm::EachProduct each_product;
         int64_t u_nnzb = 0, u_len = 0;  // add: union before the norm filter
     } plan;
     int32_t *item_order = nullptr;      // numeric processing order of the last eager multiply
@@ -293,6 +301,7 @@ struct NumericArgs {
     int32_t dtype;
     int32_t prec;
     int32_t flush_every;
+    EachProduct each_product;   // FP32 data
     // pre-split operand planes (tensor-core paths)
     const void *x_pack; const int64_t *x_pack_off;
     const void *y_pack; const int64_t *y_pack_off;

@@ -84,8 +84,8 @@ __device__ __forceinline__ void tile_run(const NumericArgs &a, ItemRun &run, int
     const unsigned before = (1u << (gi * g & 31)) - 1u;  // lanes of the groups before this one
     const int32_t shape = (m << 16) | n;
     const int xs_t = a.x_trans ? m : 1, ys_t = a.y_trans ? 1 : n;
-    // products per FP64 addition (tiny blocks always add every product)
-    const int every = a.flush_every > 0 && m * n > 16 ? a.flush_every : 1;
+    // products per FP64 addition
+    const int every = a.flush_every > 0 && !a.each_product.has(m, n) ? a.flush_every : 1;
 
     double acc[TR][TC];
     float part[TR][TC];

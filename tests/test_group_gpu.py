@@ -139,3 +139,50 @@ def test_non_finite_values_stay_in_their_rows(bsm):
     hit = np.array([(int(i), int(r)) in bad for i, r in rows])
     np.testing.assert_array_equal(got.data[~hit], base.data[~hit])
     assert not np.isfinite(got.data[hit]).all()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp64_dmma"])
+def test_fp32_sums_per_variant(bsm, prec):
+    """FP32 data with flush_every above 1: variant 1 (the default up to 16 elements, on request for 5 x 5 and 6 x 6
+    blocks) adds every product in FP64, bit for bit what flush_every = 1 gives; variant 0 adds them together."""
+    import torch
+    sizes = (2, 4, 5, 6)
+    bs = I.mixed_sizes(120, sizes, [0.25] * 4, seed=5)
+    Ah, Bh = random_bcsr(bs, bs, 0.3, seed=63, dtype=np.float32), random_bcsr(bs, bs, 0.3, seed=64, dtype=np.float32)
+    A, B = bsm.Matrix.from_host(Ah), bsm.Matrix.from_host(Bh)
+
+    def run(flush):
+        C = bsm.multiply(1.0, A, B, prec=prec, flush_every=flush)
+        g = torch.linspace(-1.0, 1.0, C.info().data_len, dtype=torch.float32, device="cuda")
+        dA, dB = (torch.empty(len(X.data), dtype=torch.float32, device="cuda") for X in (Ah, Bh))
+        bsm.multiply_backward(1.0, C, g, A, B, dA, dB, prec=prec, flush_every=flush)
+        rc = np.stack([np.repeat(bs, np.diff(C.pattern()[0])), bs[C.pattern()[1]]], 1)
+        shape = np.repeat(rc, rc[:, 0] * rc[:, 1], axis=0)
+        return C.data_host(), shape, dA.cpu().numpy(), dB.cpu().numpy()
+
+    def among(shape, keys):
+        return np.array([tuple(s) in keys for s in shape.tolist()])
+
+    try:
+        one, shape, dA1, dB1 = run(1)
+        default = run(8)[0]
+        tiny = shape[:, 0] * shape[:, 1] <= 16
+        square = among(shape, {(5, 5), (6, 6)})
+        np.testing.assert_array_equal(default[tiny], one[tiny])
+        assert (default[square] != one[square]).any()      # eight products share an FP32 sum
+        for m, n in ((5, 5), (6, 6)):
+            bsm.bsm_set_variant(prec, m, n, 1)
+        got, _, dA, dB = run(8)
+        np.testing.assert_array_equal(got[tiny | square], one[tiny | square])
+        for x, y, X in ((dA, dA1, Ah), (dB, dB1, Bh)):     # the adjoints' blocks, by their own shapes
+            rc = np.stack([np.repeat(bs, np.diff(X.row_ptr)), bs[X.col_idx]], 1)
+            s = np.repeat(rc, rc[:, 0] * rc[:, 1], axis=0)
+            keep = (s[:, 0] * s[:, 1] <= 16) | among(s, {(5, 5), (6, 6)})
+            np.testing.assert_array_equal(x[keep], y[keep])
+        bsm.bsm_set_variant(prec, 4, 4, 0)
+        got = run(8)[0]
+        four = among(shape, {(4, 4)})
+        assert (got[four] != one[four]).any()
+    finally:
+        for m, n in ((4, 4), (5, 5), (6, 6)):
+            bsm.bsm_set_variant(prec, m, n, -1)
