@@ -606,17 +606,7 @@ bsm_status ensure_transpose(bsm_mat *X) {
     if (e == cudaSuccess) e = launch_gather_i32(n, tblk, rows, trow, g_stream);
     if (e == cudaSuccess) e = launch_histogram_u32(n, keys, X->nbc, counts, g_stream);
     if (e == cudaSuccess) e = launch_scan_i64(counts, tptr, X->nbc, stmp, g_stream);
-    // the columns' bitmaps, up to 256 MB
-    const int32_t words = (X->nbr + 31) / 32;
-    uint32_t *tbits = nullptr;
-    if (e == cudaSuccess && (int64_t)X->nbc * words <= (int64_t(1) << 26)) {
-        if ((st = sc.get(&tbits, (size_t)X->nbc * words))) return st;
-        e = cudaMemsetAsync(tbits, 0, sizeof(uint32_t) * (size_t)X->nbc * words, g_stream);
-        if (e == cudaSuccess) e = launch_col_bits(n, rows, X->col_idx, words, tbits, g_stream);
-    }
     if ((st = cuda_check(e, "transpose pattern"))) return st;
-    X->t_bits = tbits;
-    if (tbits) sc.release(tbits);
     X->t_ptr = tptr;
     X->t_row = trow;
     X->t_blk = tblk;
@@ -624,6 +614,34 @@ bsm_status ensure_transpose(bsm_mat *X) {
     sc.release(trow);
     sc.release(tblk);
     return BSM_OK;
+}
+
+// Whether the fill of `nprod` products goes through bitmaps of B's columns, a word
+// for every 32 inner blocks.  Per C block the bitmaps read two words and expand one
+// per word of the inner dimension, and the walk reads the column's blocks twice; the
+// bitmaps' set-up is worth some 48 blocks of the walk.  Fill phase in ms, walk and
+// bitmaps, by words and blocks per column, random and banded columns:
+//   32 words   64: 4.0 and 4.0, 0.92 and 1.14   96: 6.6 and 4.6, 1.88 and 1.89
+//   125        144: 9.2 and 10.3, 1.08 and 1.38   224: 16.3 and 11.4, 2.36 and 2.33
+//   375        320: 6.6 and 8.4, 0.74 and 0.91   448: 10.8 and 9.4, 1.38 and 1.28
+//   938        100: 20.1 and 113, 23.3 and 135   1000: 16.2 and 16.9, 2.34 and 1.98
+// Below 4e6 products the difference is under 0.1 ms, less than making them.  By the
+// rule they take less than 4 bytes per block of B; they stay on the handle while its
+// pattern does, up to 256 MB.
+bool fill_bitmaps(const bsm_mat *B, int64_t nprod, int32_t nwords, int64_t max_ccnt) {
+    const int64_t words = ((int64_t)B->nbr + 31) / 32 * B->nbc;
+    return nprod >= (int64_t(1) << 22) && B->nnzb >= words + 48 * (int64_t)B->nbc && words <= (int64_t(1) << 26) &&
+           symbolic_fill_cols_smem_bytes(nwords, (int32_t)max_ccnt, B->nbr, true) <= 200 * 1024;
+}
+
+bsm_status ensure_col_bits(bsm_mat *X) {
+    if (X->t_bits) return BSM_OK;
+    uint32_t *bits = nullptr;
+    if (const bsm_status st = dalloc_t(&bits, ((size_t)X->nbr + 31) / 32 * X->nbc)) return st;
+    const bsm_status st = cuda_check(launch_col_bits(X, bits, g_stream), "column bitmaps");
+    if (st) dfree(bits);
+    else X->t_bits = bits;
+    return st;
 }
 
 bsm_status read_words(const int64_t *const *src, int n) {
@@ -1418,12 +1436,6 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
 
     // ---- a2: symbolic count
     SymbolicArgs sa{};
-    if (use_filter) {
-        double *b_min;
-        if ((st = sc.get(&b_min, 1))) return st;
-        if ((st = cuda_check(launch_min_norm(B->nnzb, nB, b_min, g_stream), "smallest norm"))) return st;
-        sa.b_min = b_min;
-    }
     sa.nbr = nbr; sa.nbk = nbk; sa.nbc = nbc;
     sa.a_row_bs = A->row_bs; sa.a_col_bs = A->col_bs; sa.a_row_ptr = A->row_ptr; sa.a_col_idx = A->col_idx;
     sa.a_norm = nA;
@@ -1549,17 +1561,28 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
     }
     FillOut fo{prod_ptr, crow_ptr, celem_ptr, c_col, c_off, c_rc, cptr, pa, pb, pc, old_off, (int32_t)max_ccnt, nchunk};
     // fill through B's columns when the k -> A block map fits in shared memory
-    const bool by_cols = symbolic_fill_cols_smem_bytes(nwords, (int32_t)max_ccnt, nbk) <= 200 * 1024;
+    const bool by_cols = symbolic_fill_cols_smem_bytes(nwords, (int32_t)max_ccnt, nbk, false) <= 200 * 1024;
+    const uint32_t *col_bits = nullptr;
     if (by_cols) {
         if (no_sync && !B->t_ptr) return set_error(BSM_ERR_ARG, "no_sync: B's column copy is missing");
         if ((st = ensure_transpose(B))) return st;
+        if (fill_bitmaps(B, nprod, nwords, max_ccnt)) {
+            if (!no_sync && (st = ensure_col_bits(B))) return st;
+            col_bits = B->t_bits;
+        }
+    }
+    if (col_bits && use_filter) {
+        double *b_min;
+        if ((st = sc.get(&b_min, 1))) return st;
+        if ((st = cuda_check(launch_min_norm(B->nnzb, nB, b_min, g_stream), "smallest norm"))) return st;
+        sa.b_min = b_min;
     }
     // rows [r0, r1) of C's pattern and of the product list (offsets relative to prod_ptr[r0])
     auto fill_rows = [&](int32_t r0, int32_t r1, int64_t prod_base) -> cudaError_t {
         FillOut f = fo;
         f.row0 = r0;
         f.prod_base = prod_base;
-        return by_cols ? launch_symbolic_fill_cols(sa, bitmaps, f, B->t_ptr, B->t_row, B->t_blk, B->t_bits, g_stream,
+        return by_cols ? launch_symbolic_fill_cols(sa, bitmaps, f, B->t_ptr, B->t_row, B->t_blk, col_bits, g_stream,
                                                  r1 - r0)
                        : launch_symbolic_fill(sa, bitmaps, f, g_stream, r1 - r0);
     };

@@ -124,7 +124,7 @@ struct bsm_mat {
     // column-major copy of the pattern (built on demand, dropped with the pattern)
     int64_t *t_ptr = nullptr;           // [nbc+1]
     int32_t *t_row = nullptr, *t_blk = nullptr;  // [nnzb]
-    uint32_t *t_bits = nullptr;         // [nbc * ceil(nbr / 32)] block rows of every column (null: too large)
+    uint32_t *t_bits = nullptr;         // [nbc * ceil(nbr / 32)] block rows of every column (null: not built)
 
     // provenance of the last bsm_add that wrote this matrix (for its adjoint):
     // per block, the element offset of the matching X / Y block or -1
@@ -187,7 +187,7 @@ struct SymbolicArgs {
     int use_filter;
     int32_t nwords;                      // ceil(nbc / 32)
     const int32_t *status;               // nullable: kernels that read it do nothing when *status != 0
-    const double *b_min;                 // smallest norm of B (with the filter), 0 where one is NaN
+    const double *b_min;                 // smallest norm of B (filter and column bitmaps), 0 where one is NaN
 };
 
 // Per block row: kept products, distinct C columns, C elements; bitmaps of
@@ -220,12 +220,11 @@ int64_t symbolic_fill_smem_bytes(int32_t nwords, int32_t max_ccnt, int nchunk);
 cudaError_t launch_symbolic_fill_cols(const SymbolicArgs &a, const uint32_t *bitmaps, const FillOut &o,
                                       const int64_t *bt_ptr, const int32_t *bt_k, const int32_t *bt_b,
                                       const uint32_t *bt_bits, cudaStream_t s, int32_t nrows = -1);
-int64_t symbolic_fill_cols_smem_bytes(int32_t nwords, int32_t max_ccnt, int32_t nbk);
-// *out = smallest of n norms, 0 where one is NaN (n = 0: +infinity)
+int64_t symbolic_fill_cols_smem_bytes(int32_t nwords, int32_t max_ccnt, int32_t nbk, bool bits);
+// *out = smallest of n norms and 1.4e306, 0 where one is NaN
 cudaError_t launch_min_norm(int64_t n, const double *norms, double *out, cudaStream_t s);
-// bits[col][row / 32] |= 1 << row % 32 for every block (bits zeroed by the caller; words = ceil(nbr / 32))
-cudaError_t launch_col_bits(int64_t n, const int32_t *rows, const int32_t *cols, int32_t words, uint32_t *bits,
-                            cudaStream_t s);
+// bits[col][row / 32] of X's blocks, ceil(nbr / 32) words per column
+cudaError_t launch_col_bits(const bsm_mat *X, uint32_t *bits, cudaStream_t s);
 cudaError_t launch_blk_rows(const bsm_mat *X, int32_t *rows, cudaStream_t s);
 
 // Stable LSD radix sort of (key, value) pairs by the low `key_bits` bits.

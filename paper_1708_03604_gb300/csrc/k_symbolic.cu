@@ -395,9 +395,13 @@ __global__ void __launch_bounds__(kThreads) k_min_norm(int64_t n, const double *
     if (threadIdx.x == 0) atomicMin(out, part);
 }
 
-__global__ void k_col_bits(int64_t n, const int32_t *rows, const int32_t *cols, int32_t words, uint32_t *bits) {
-    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n; b += (int64_t)gridDim.x * blockDim.x)
-        atomicOr(&bits[(int64_t)cols[b] * words + (rows[b] >> 5)], 1u << (rows[b] & 31));
+// one warp per block row
+__global__ void k_col_bits(int32_t nbr, const int64_t *row_ptr, const int32_t *col_idx, int32_t words, uint32_t *bits) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < nbr; i += nwarp)
+        for (int64_t b = row_ptr[i] + lane; b < row_ptr[i + 1]; b += 32)
+            atomicOr(&bits[(int64_t)col_idx[b] * words + (i >> 5)], 1u << (i & 31));
 }
 
 // Fill through B's columns.  Same outputs as k_sym_fill, but every C block
@@ -405,12 +409,14 @@ __global__ void k_col_bits(int64_t n, const int32_t *rows, const int32_t *cols, 
 // products come out in ascending k already and are written contiguously
 // (coalesced) instead of scattered across the row's C blocks.
 //
-// Where the filter can drop nothing of the row (no threshold, or the smallest
-// norms multiplied exceed it) the kept products of (i, j) are the common bits of
-// row i of A and column j of B: counting them reads a bit per inner block, and
-// the blocks' indices are ranks in the two bitmaps.  Elsewhere the column is
-// walked against a shared-memory map k -> A block of row i.  3,000 block rows of
-// 5/13/23 (2.5e8 products): the walk 8.6 ms, the bitmaps 2.5.
+// With B's column bitmaps, where the filter can drop nothing of the row (no
+// threshold, or the smallest norms multiplied exceed it) the kept products of (i,
+// j) are the common bits of row i of A and column j of B: counting them reads a
+// bit per inner block, and the blocks' indices are ranks in the two bitmaps.
+// Elsewhere the column is walked against a shared-memory map k -> A block of row
+// i.  The bitmaps cost by the inner dimension and the walk by the column's length
+// (fill_bitmaps, which decides); 3,000 block rows of 5/13/23 (2.5e8 products): the
+// walk 8.6 ms, the bitmaps 2.5.
 constexpr int kFillWords = 32;                    // bitmap words a warp expands at a time
 struct FillWarp {
     uint16_t list[kFillWords * 32];               // k of the products, relative to the first word
@@ -941,10 +947,12 @@ int64_t symbolic_fill_smem_bytes(int32_t nwords, int32_t max_ccnt, int nchunk) {
     return (2 * (int64_t)nwords + (int64_t)(nchunk + 1) * max_ccnt + 1) * (int64_t)sizeof(int32_t);
 }
 
-int64_t symbolic_fill_cols_smem_bytes(int32_t nwords, int32_t max_ccnt, int32_t nbk) {
-    // the map k -> A block, or row i's bitmap and ranks and the warps' lists
-    const int64_t map = std::max<int64_t>(nbk, 2 * (((int64_t)nbk + 31) / 32) +
-                                                   (int64_t)(kThreads / 32 * sizeof(FillWarp) / sizeof(int32_t)));
+int64_t symbolic_fill_cols_smem_bytes(int32_t nwords, int32_t max_ccnt, int32_t nbk, bool bits) {
+    // the map k -> A block; with the bitmaps, row i's bitmap and ranks and the warps' lists in its place
+    int64_t map = nbk;
+    if (bits)
+        map = std::max<int64_t>(nbk, 2 * (((int64_t)nbk + 31) / 32) +
+                                         (int64_t)(kThreads / 32 * sizeof(FillWarp) / sizeof(int32_t)));
     return (2 * (int64_t)nwords + (int64_t)max_ccnt + map + 1) * (int64_t)sizeof(int32_t);
 }
 
@@ -957,10 +965,11 @@ cudaError_t launch_min_norm(int64_t n, const double *norms, double *out, cudaStr
     return cudaGetLastError();
 }
 
-cudaError_t launch_col_bits(int64_t n, const int32_t *rows, const int32_t *cols, int32_t words, uint32_t *bits,
-                            cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    k_col_bits<<<grid_for(n), kThreads, 0, s>>>(n, rows, cols, words, bits);
+cudaError_t launch_col_bits(const bsm_mat *X, uint32_t *bits, cudaStream_t s) {
+    const int32_t words = (X->nbr + 31) / 32;
+    cudaError_t e = cudaMemsetAsync(bits, 0, sizeof(uint32_t) * (size_t)X->nbc * words, s);
+    if (e != cudaSuccess || X->nnzb == 0) return e;
+    k_col_bits<<<grid_for((int64_t)X->nbr * 32), kThreads, 0, s>>>(X->nbr, X->row_ptr, X->col_idx, words, bits);
     count_launch(1);
     return cudaGetLastError();
 }
@@ -970,7 +979,7 @@ cudaError_t launch_symbolic_fill_cols(const SymbolicArgs &a, const uint32_t *bit
                                       const uint32_t *bt_bits, cudaStream_t s, int32_t nrows) {
     if (nrows < 0) nrows = a.nbr - o.row0;
     if (nrows <= 0) return cudaSuccess;
-    const int smem = (int)symbolic_fill_cols_smem_bytes(a.nwords, o.max_ccnt, a.nbk);
+    const int smem = (int)symbolic_fill_cols_smem_bytes(a.nwords, o.max_ccnt, a.nbk, bt_bits != nullptr);
     if (const cudaError_t e = allow_dynamic_smem(k_sym_fill_cols, smem)) return e;
     k_sym_fill_cols<<<nrows, kThreads, smem, s>>>(a, bitmaps, o, bt_ptr, bt_k, bt_b, bt_bits);
     count_launch(1);
