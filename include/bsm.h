@@ -422,7 +422,8 @@ bsm_status bsm_block_norms(bsm_t X, double *out);
  *   B keeps a column-major copy of its pattern until that changes and, where
  *   its columns are long enough for them (on average a block per 32 block rows
  *   and 48 more, 4e6 products), a bitmap of every column: less than 4 bytes per
- *   block of B and at most 256 MB.
+ *   block of B and at most 256 MB.  Where their memory is refused the multiply
+ *   goes on without them.
  */
 bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C,
                         double filter_eps, const bsm_opts *opts);

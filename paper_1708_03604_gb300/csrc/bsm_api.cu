@@ -634,10 +634,16 @@ bool fill_bitmaps(const bsm_mat *B, int64_t nprod, int32_t nwords, int64_t max_c
            symbolic_fill_cols_smem_bytes(nwords, (int32_t)max_ccnt, B->nbr, true) <= 200 * 1024;
 }
 
+// The bitmaps are optional: where their memory is refused t_bits stays null and
+// the columns are walked.
 bsm_status ensure_col_bits(bsm_mat *X) {
     if (X->t_bits) return BSM_OK;
+    const std::string before = t_err;
     uint32_t *bits = nullptr;
-    if (const bsm_status st = dalloc_t(&bits, ((size_t)X->nbr + 31) / 32 * X->nbc)) return st;
+    if (dalloc_t(&bits, ((size_t)X->nbr + 31) / 32 * X->nbc) != BSM_OK) {
+        t_err = before;
+        return BSM_OK;
+    }
     const bsm_status st = cuda_check(launch_col_bits(X, bits, g_stream), "column bitmaps");
     if (st) dfree(bits);
     else X->t_bits = bits;

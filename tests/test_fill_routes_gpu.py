@@ -89,3 +89,9 @@ def test_few_products_are_walked(bsm, oracle):
     bs = I.uniform_sizes(200, 1)
     Ah, Bh = random_bcsr(bs, I.uniform_sizes(70, 1), 0.5, seed=95), random_bcsr(I.uniform_sizes(70, 1), bs, 0.5, seed=96)
     assert _bitmap_bytes(Bh) not in _check(bsm, oracle, Ah, Bh, 0.0)
+
+
+def test_refused_bitmaps_fall_back_to_the_walk(bsm, oracle):
+    Ah, Bh = random_bcsr(I.uniform_sizes(1024, 1), I.uniform_sizes(1024, 1), 0.1, seed=97), _columns(1024, 1030, 90, 98)
+    for eps in (0.0, 1e-9):
+        assert _bitmap_bytes(Bh) in _check(bsm, oracle, Ah, Bh, eps, refuse=_bitmap_bytes(Bh))
