@@ -5,18 +5,21 @@ the knobs of this library's kernels).
 What it searches, per precision, by timing the numeric kernel (CUDA events
 recorded by the library around the launch) on the caller's operands:
 
-* per output block shape (m, n): the variant -- one warp per block (FP64:
-  lanes over its elements; split and Ozaki paths: tensor-core MMAs on packed
-  fragments) or, for blocks of at most 16 elements and 5 x 5 ones (FP64 and
-  Ozaki also 6 x 6), one lane per block on the CUDA cores;
+* per output block shape (m, n) of the FP64_DMMA, split and Ozaki paths: the
+  variant -- one warp per block (FP64_DMMA: lanes over its elements; split and
+  Ozaki paths: tensor-core MMAs on packed fragments) or, for blocks of at most
+  16 elements and 5 x 5 ones (FP64_DMMA and Ozaki also 6 x 6), the CUDA cores,
+  one lane per block or, on the split paths, per element (BSM_P_FP64 and FP32
+  data choose the lanes of a block themselves: no search, the library's
+  variants are recorded);
 * the FP64 FMA kernel build (how many output elements a lane holds per pass:
-  up to 13 or up to 24) -- BSM_P_FP64;
+  up to 13 or up to 24) -- BSM_P_FP64 on FP64 data;
 * warps per CTA (4 or 2) of the persistent mma.sync kernels;
 * persistent CTAs per SM;
 * the fragment-tile pass shape (tiles along rows and columns that one pass
   over a block's products covers) of the split, Ozaki and FP64-MMA kernels
-  (on the split paths also the default split: blocks of one tile row in a
-  kernel instance of their own, compiled for 1-row passes);
+  (on the split paths also the default: a kernel instance per height class of
+  the blocks);
 * the order of the output blocks: by block row, or by 2-D tiles of ranked
   rows x ranked columns so that the blocks in flight share A's and B's
   blocks in L2;
@@ -105,16 +108,19 @@ def tune(A: bsm.Matrix, B: bsm.Matrix, eps: float = 0.0, prec: str = "tf32x3", r
     fp64_like = prec in ("fp64", "fp64_dmma", "ozaki")  # lane variant = plain FP64 FMA
     shapes = [(m, n) for m, n in _shapes(A, B)
               if m * n <= 16 or (m, n) == (5, 5) or (fp64_like and (m, n) == (6, 6))]
+    # the CUDA-core kernels of these precisions choose the lanes of a block themselves
+    fp32 = A.info().dtype == bsm.BSM_FP32 and prec in ("fp64", "fp64_dmma")
+    searched = [] if fp32 or prec == "fp64" else shapes
     reset(prec)
     for m, n in shapes:
-        bsm.bsm_set_variant(prec, m, n, 0)
+        bsm.bsm_set_variant(prec, m, n, 0 if searched else -1)
     Cm = bsm.Matrix.empty(A.row_bs, B.col_bs)
     bsm.bsm_set_profiling(True)
     try:
         _numeric_ms(A, B, eps, prec, 1, Cm)  # warm-up
         start = best = _numeric_ms(A, B, eps, prec, reps, Cm)
-        variants = {}
-        for m, n in shapes:
+        variants = {f"{m}x{n}": bsm.bsm_get_variant(prec, m, n) for m, n in shapes}
+        for m, n in searched:
             bsm.bsm_set_variant(prec, m, n, 1)
             t = _numeric_ms(A, B, eps, prec, reps, Cm)
             if t < best * (1.0 - gain):
@@ -122,11 +128,12 @@ def tune(A: bsm.Matrix, B: bsm.Matrix, eps: float = 0.0, prec: str = "tf32x3", r
                 variants[f"{m}x{n}"] = 1
             else:
                 bsm.bsm_set_variant(prec, m, n, 0)
-                variants[f"{m}x{n}"] = 0
         params = {}
         for name, values in SEARCH.get(prec, []):
             if name == "engine":
                 continue       # decided last, on the whole multiply's time
+            if fp32 and name not in ("ctas_per_sm", "sched_tile"):
+                continue       # the FP32 tile kernel has no such knob
             chosen = values[0]
             bsm.bsm_set_tuning(prec, name, chosen)
             for v in values[1:]:
