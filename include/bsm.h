@@ -298,7 +298,8 @@ enum {
     BSM_K_PANEL_TCGEN05 = 4
 };
 /* What the last numeric launch into C ran: cfg[0] kernel (BSM_K_*),
- * cfg[1] FP64 kernel build (0 small, 1 narrow, 2 wide; -1 for the others),
+ * cfg[1] build of the FP64 FMA kernel (0 small, 1 narrow, 2 wide; -1 for the
+ * other kernels and for FP32 data),
  * cfg[2] threads per CTA, cfg[3] CTAs, cfg[4] / cfg[5] fragment tiles per pass
  * along rows / columns (0 where the kernel has no passes; cfg[4] = 0 on the
  * split paths when one-tile-row blocks ran in their own instance, cfg[3] then

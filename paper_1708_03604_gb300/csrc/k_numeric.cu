@@ -1206,16 +1206,20 @@ cudaError_t launch_numeric(const NumericArgs &args, cudaStream_t s, NumericLaunc
         li = NumericLaunch{BSM_K_FP64_MMA, -1, kThreadsNum, grid, a.pass_mt > 0 ? a.pass_mt : 3,
                            a.pass_nt > 0 ? a.pass_nt : 3};
     } else if (!tc) {
-        // the build by the largest output block: all within one narrow pass
-        // (<= 288 elements) or beyond the wide ladder's single pass (> 768)
-        // run narrow -- measured faster there -- the rest wide; the tuner may
-        // ask for narrow or wide instead (the small build only ever runs when
-        // every output block has at most 16 elements)
-        const int area = a.max_out_rows * a.max_out_cols;
-        int build = (area > 0 && area <= 16) ? kCcSmall : (area <= 288 || area > 768) ? kCcNarrow : kCcWide;
-        if (a.fp64_build == 1 && build != kCcSmall) build = kCcNarrow;
-        if (a.fp64_build == 2 && build != kCcSmall) build = kCcWide;
+        int build = -1;
         if (a.dtype == BSM_FP64) {
+            // the build by the largest output block: narrow up to 288 elements and
+            // beyond the wide ladder's single pass (768), wide between, where its
+            // larger Q fill more lane slots; narrow and wide in ms (3e10 useful
+            // FLOP, 10% occupancy): 16 x 16 23.9 and 24.3, 17 x 17 27.4 and 25.6,
+            // 18 x 18 26.2 and 25.1, 20 x 20 25.0 and 25.1, 23 x 23 26.1 and 24.8,
+            // 24 x 24 24.0 and 24.2, 32 x 32 24.5 and 24.7.  The tuner may ask for
+            // either; the small build only ever runs when every output block has at
+            // most 16 elements
+            const int area = a.max_out_rows * a.max_out_cols;
+            build = (area > 0 && area <= 16) ? kCcSmall : (area <= 288 || area > 768) ? kCcNarrow : kCcWide;
+            if (a.fp64_build == 1 && build != kCcSmall) build = kCcNarrow;
+            if (a.fp64_build == 2 && build != kCcSmall) build = kCcWide;
             e = launch_numeric_group(a, build, s, &grid);
         } else {
             e = launch_numeric_tile(a, s, &grid);

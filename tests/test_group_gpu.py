@@ -186,3 +186,13 @@ def test_fp32_sums_per_variant(bsm, prec):
     finally:
         for m, n in ((4, 4), (5, 5), (6, 6)):
             bsm.bsm_set_variant(prec, m, n, -1)
+
+
+def test_fp32_reports_no_fp64_build(bsm):
+    """The launch configuration names a build for FP64 data only."""
+    bs = I.mixed_sizes(60, (5, 13), (0.5, 0.5), seed=9)
+    Ah = random_bcsr(bs, bs, 0.2, seed=74)
+    for X, build in ((Ah, 1), (Ah.astype(np.float32), -1)):
+        A = bsm.Matrix.from_host(X)
+        cfg = bsm.multiply(1.0, A, A).launch_config()
+        assert cfg["kernel"] == "fp64_cores" and cfg["fp64_build"] == build and cfg["grid"] > 0
