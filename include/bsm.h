@@ -244,17 +244,17 @@ bsm_status bsm_get_variant(int32_t prec, int32_t m, int32_t n, int32_t *variant)
  *                        0 = as many as fit (default)
  *   BSM_TUNE_PASS_MT     fragment tiles along the output rows per pass over
  *                        a block's products: split paths 1..2 (16-row tiles;
- *                        default: output blocks of one tile row run in a
- *                        kernel instance compiled for 1-row passes -- fewer
- *                        registers, more warps per SM -- and the others in a
- *                        2-row instance, two launches; 1 or 2 runs every block
- *                        in that one instance), FP64_DMMA 1..3 (default 3,
- *                        8-row tiles)
+ *                        default: a kernel instance per height class of the
+ *                        output blocks, over 24 rows, 17 to 24, 9 to 16 and at
+ *                        most 8 -- fewer registers, more warps per SM -- one
+ *                        launch each; 1 or 2 runs every block in one instance
+ *                        for any height), FP64_DMMA 1..3 (default 3, 8-row
+ *                        tiles)
  *   BSM_TUNE_PASS_NT     along the columns: split paths 1..3 (default 3,
  *                        8-column tiles), OZAKI 1..3 (default 3; 1 and 2 run
  *                        a kernel instance with a smaller staging ring and
  *                        fewer registers), FP64_DMMA 1..3 (default 3)
- *   BSM_TUNE_FP64_BUILD  BSM_P_FP64 only: FP64 FMA kernel build, 0 chosen by
+ *   BSM_TUNE_FP64_BUILD  BSM_P_FP64 on FP64 data: FMA kernel build, 0 chosen by
  *                        the largest output block (default), 1 narrow (up to
  *                        13 elements per lane per pass), 2 wide (up to 24);
  *                        output blocks of at most 16 elements always run the
@@ -302,8 +302,8 @@ enum {
  * other kernels and for FP32 data),
  * cfg[2] threads per CTA, cfg[3] CTAs, cfg[4] / cfg[5] fragment tiles per pass
  * along rows / columns (0 where the kernel has no passes; cfg[4] = 0 on the
- * split paths when one-tile-row blocks ran in their own instance, cfg[3] then
- * the CTAs of the 2-row instance). */
+ * split paths when every height class ran in its own instance, cfg[3] then the
+ * CTAs of the first). */
 bsm_status bsm_get_launch_config(bsm_t C, int32_t *cfg);
 
 /* Fills `opts` with the defaults (FP64, no post filter, stacks built). */

@@ -265,7 +265,6 @@ bsm_status check_opts(const bsm_opts *o, bsm_opts *out) {
 bool is_tc(int prec) {
     return prec == BSM_P_TF32x3 || prec == BSM_P_BF16x3 || prec == BSM_P_BF16x6 || prec == BSM_P_OZAKI;
 }
-// split paths whose lane variant multiplies unpacked FP32 pieces
 // the kernel instances that output blocks of these heights and products of these
 // inner sizes need
 void tile_masks(const std::vector<int32_t> &rows, const std::vector<int32_t> &inner, NumericArgs &na) {
@@ -276,6 +275,7 @@ void tile_masks(const std::vector<int32_t> &rows, const std::vector<int32_t> &in
     }
 }
 
+// split paths whose lane variant multiplies unpacked FP32 pieces
 bool needs_plain(int prec) { return is_tc(prec) && prec != BSM_P_OZAKI; }
 
 // first global row / column of every block row / column, on the device

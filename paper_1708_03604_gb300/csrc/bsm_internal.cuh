@@ -346,7 +346,7 @@ struct NumericLaunch {
     int32_t cta_threads, grid, pass_mt, pass_nt;
 };
 cudaError_t launch_numeric(const NumericArgs &a, cudaStream_t s, NumericLaunch *info = nullptr);
-// Builds of the CUDA-core kernels by the largest output block (elements a lane holds)
+// Builds of the FP64 FMA kernel by the largest output block (elements a lane holds)
 constexpr int kCcSmall = 0, kCcNarrow = 1, kCcWide = 2;
 // FP64 data on the CUDA cores (k_group.cu); *grid: CTAs launched
 cudaError_t launch_numeric_group(const NumericArgs &a, int build, cudaStream_t s, int *grid);
@@ -361,7 +361,7 @@ uint32_t split_bf16x3_debug_bits(cudaStream_t s);
 uint32_t split_bf16x6_debug_bits(cudaStream_t s);
 uint32_t tile_debug_bits(cudaStream_t s);
 int num_sms();
-// out[g] = number of keys below thr[g] in the ascending keys[0..n) (g < 2)
+// out[g] = number of keys below thr[g] in the ascending keys[0..n)
 cudaError_t launch_group_bounds(const uint32_t *keys, int64_t n, const uint32_t (&thr)[kSplitGroups - 1], int64_t *out,
                                 cudaStream_t s);
 

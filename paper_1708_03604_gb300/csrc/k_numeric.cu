@@ -490,9 +490,13 @@ __device__ __forceinline__ void oz_step(float (&acc)[kOzLevels][NTC][4], const u
 // staged through a ring laid out for passes of at most MAXN tiles.  HM: half a tile
 // of rows; HKS: some product has an HK step (the multiply's inner sizes tell).
 //
-// Bound by the tensor pipe (61% busy with two CTAs of four warps an SM, which is
-// what the accumulators leave room for) and the L2 reads, 15 chunks of 512 bytes to
-// 63 MMAs.  Blocks of 23 end in half a tile both ways: four whole steps a product,
+// Bound by the latency of a warp's steps at eight warps an SM: 2,000 banded rows of
+// 23, the kernels of the half and of the whole tile rows, tensor pipe 42% and 48%
+// busy, issue 35% and 32%.  Two CTAs of four warps fit, in the whole-row kernel by
+// its 200 registers, in the half-row one by its staging ring of 90 KB (with 166
+// registers three would; half a tile row needs 12 of the ring's 24 X words a lane).
+// Then the L2 reads, 15 chunks of 512 bytes to the 63 MMAs of a whole step.
+// Blocks of 23 end in half a tile both ways: four whole steps a product,
 // 252 MMAs and 60 chunks, became 159 and 40.5.  Numeric pass of 2,000 banded rows
 // of 23 (1.96e7 products) 55.0 -> 47.5 ms, of blocks of 5 (8e7) 26.0 -> 19.8, of 13
 // (6.9e6) 7.34 -> 7.16, of 32 (4.6e5) 4.44 -> 4.13, the last two from the running
