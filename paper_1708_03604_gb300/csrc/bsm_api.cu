@@ -246,6 +246,7 @@ void free_pattern(bsm_mat *X) {
     dfree(X->t_row); X->t_row = nullptr;
     dfree(X->t_blk); X->t_blk = nullptr;
     dfree(X->t_bits); X->t_bits = nullptr;
+    X->rewritten = false;
     X->nnzb = 0;
     X->data_len = 0;
 }
@@ -582,20 +583,22 @@ bsm_status shape_order(Scratch &sc, int64_t n, const int32_t *blk_rc, const std:
 
 // Column-major copy of X's pattern (kept on the handle until its pattern
 // changes): t_ptr[nbc+1], and for every block in column order (ascending
-// block row inside a column) its block row t_row and block index t_blk.
+// block row inside a column) its block row t_row and block index t_blk.  Made
+// again, in its place, where a no-sync call may have written another pattern.
 bsm_status ensure_transpose(bsm_mat *X) {
-    if (X->t_ptr) return BSM_OK;
+    if (X->t_ptr && !X->rewritten) return BSM_OK;
     Scratch sc;
     bsm_status st;
     const int64_t n = X->nnzb;
     int32_t *rows, *iota, *vals_alt;
     uint32_t *keys, *keys_alt, *keys_sorted;
-    int64_t *rtmp, *counts, *stmp, *tptr;
-    int32_t *trow, *tblk;
+    int64_t *rtmp, *counts, *stmp, *tptr = X->t_ptr;
+    int32_t *trow = X->t_row, *tblk = X->t_blk;
     if ((st = sc.get(&rows, n)) || (st = sc.get(&iota, n)) || (st = sc.get(&vals_alt, n)) || (st = sc.get(&keys, n)) ||
         (st = sc.get(&keys_alt, n)) || (st = sc.get(&keys_sorted, n)) || (st = sc.get(&rtmp, radix_tmp_elems(n))) ||
-        (st = sc.get(&counts, X->nbc)) || (st = sc.get(&stmp, scan_tmp_elems(X->nbc))) ||
-        (st = sc.get(&tptr, (size_t)X->nbc + 1)) || (st = sc.get(&trow, n)) || (st = sc.get(&tblk, n)))
+        (st = sc.get(&counts, X->nbc)) || (st = sc.get(&stmp, scan_tmp_elems(X->nbc))))
+        return st;
+    if (!tptr && ((st = sc.get(&tptr, (size_t)X->nbc + 1)) || (st = sc.get(&trow, n)) || (st = sc.get(&tblk, n))))
         return st;
     int bits = 1;
     while ((1ll << bits) < (int64_t)X->nbc) ++bits;
@@ -637,7 +640,8 @@ bool fill_bitmaps(const bsm_mat *B, int64_t nprod, int32_t nwords, int64_t max_c
 // The bitmaps are optional: where their memory is refused t_bits stays null and
 // the columns are walked.
 bsm_status ensure_col_bits(bsm_mat *X) {
-    if (X->t_bits) return BSM_OK;
+    if (X->t_bits)
+        return X->rewritten ? cuda_check(launch_col_bits(X, X->t_bits, g_stream), "column bitmaps") : BSM_OK;
     const std::string before = t_err;
     uint32_t *bits = nullptr;
     if (dalloc_t(&bits, ((size_t)X->nbr + 31) / 32 * X->nbc) != BSM_OK) {
@@ -1571,7 +1575,13 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
     const uint32_t *col_bits = nullptr;
     if (by_cols) {
         if (no_sync && !B->t_ptr) return set_error(BSM_ERR_ARG, "no_sync: B's column copy is missing");
-        if ((st = ensure_transpose(B))) return st;
+        if (!no_sync && (st = ensure_transpose(B))) return st;
+        // B an output: a no-sync call may have given it another pattern of its size
+        if (no_sync && B->plan.kind != 0) {
+            int32_t *stale = reinterpret_cast<int32_t *>(totals + 3);  // zeroed with the totals
+            if ((st = cuda_check(launch_check_columns(B, stale, g_stream), "column copy"))) return st;
+            sa.stale = stale;
+        }
         if (fill_bitmaps(B, nprod, nwords, max_ccnt)) {
             if (!no_sync && (st = ensure_col_bits(B))) return st;
             col_bits = B->t_bits;
@@ -1588,9 +1598,14 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
         FillOut f = fo;
         f.row0 = r0;
         f.prod_base = prod_base;
-        return by_cols ? launch_symbolic_fill_cols(sa, bitmaps, f, B->t_ptr, B->t_row, B->t_blk, col_bits, g_stream,
-                                                 r1 - r0)
-                       : launch_symbolic_fill(sa, bitmaps, f, g_stream, r1 - r0);
+        if (!by_cols) return launch_symbolic_fill(sa, bitmaps, f, g_stream, r1 - r0);
+        cudaError_t fe = launch_symbolic_fill_cols(sa, bitmaps, f, B->t_ptr, B->t_row, B->t_blk, col_bits, g_stream, r1 - r0);
+        if (fe == cudaSuccess && sa.stale) {
+            SymbolicArgs by_rows = sa;
+            by_rows.when_stale = 1;
+            fe = launch_symbolic_fill(by_rows, bitmaps, f, g_stream, r1 - r0);
+        }
+        return fe;
     };
     if (!chunked) {  // a chunked multiply fills each row panel right before its numeric pass
         e = fill_rows(0, nbr, 0);
@@ -1810,7 +1825,10 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
     }
     ev.mark(6);
     }
-    if (no_sync) return BSM_OK;  // C's storage, counts and plan are unchanged
+    if (no_sync) {  // C's storage, counts and plan are unchanged
+        C->rewritten = true;
+        return BSM_OK;
+    }
 
     // ---- swap C's pattern (old arrays are freed stream-ordered after the numeric kernel)
     free_results(C);
@@ -2189,6 +2207,7 @@ bsm_status bsm_add(double a, bsm_t X, double b, bsm_t Y, bsm_t Z, double filter_
     if (e == cudaSuccess) e = launch_add_values(nnz, zo, zrc, xs, ys, a, X->data, b, Y->data, zd, X->dtype, stat, g_stream);
     if (e == cudaSuccess && direct) e = launch_copy_i64_if_ok(nbr + 1, zrow, Z->row_ptr, Z->status, g_stream);
     if ((st = cuda_check(e, "add fill"))) return st;
+    if (no_sync) Z->rewritten = true;
     if (direct) return BSM_OK;
     if (no_sync) {
         // filter the union (scratch) into Z's storage; its row pointers are

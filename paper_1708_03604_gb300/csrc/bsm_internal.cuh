@@ -125,6 +125,9 @@ struct bsm_mat {
     int64_t *t_ptr = nullptr;           // [nbc+1]
     int32_t *t_row = nullptr, *t_blk = nullptr;  // [nnzb]
     uint32_t *t_bits = nullptr;         // [nbc * ceil(nbr / 32)] block rows of every column (null: not built)
+    // a no-sync call has written the pattern, and a graph may do so again unseen by
+    // the host: the copies above may be those of an earlier pattern of the same size
+    bool rewritten = false;
 
     // provenance of the last bsm_add that wrote this matrix (for its adjoint):
     // per block, the element offset of the matching X / Y block or -1
@@ -188,6 +191,10 @@ struct SymbolicArgs {
     int32_t nwords;                      // ceil(nbc / 32)
     const int32_t *status;               // nullable: kernels that read it do nothing when *status != 0
     const double *b_min;                 // smallest norm of B (filter and column bitmaps), 0 where one is NaN
+    // nullable: the kernel runs only where *stale != 0 is when_stale (B's column copy
+    // is not that of its pattern: fill by rows)
+    const int32_t *stale;
+    int32_t when_stale;
 };
 
 // Per block row: kept products, distinct C columns, C elements; bitmaps of
@@ -223,6 +230,8 @@ cudaError_t launch_symbolic_fill_cols(const SymbolicArgs &a, const uint32_t *bit
 int64_t symbolic_fill_cols_smem_bytes(int32_t nwords, int32_t max_ccnt, int32_t nbk, bool bits);
 // *out = smallest of n norms and 1.4e306, 0 where one is NaN
 cudaError_t launch_min_norm(int64_t n, const double *norms, double *out, cudaStream_t s);
+// *stale = 1 where the column copy is not the one of X's pattern (of the same size); zeroed by the caller
+cudaError_t launch_check_columns(const bsm_mat *X, int32_t *stale, cudaStream_t s);
 // bits[col][row / 32] of X's blocks, ceil(nbr / 32) words per column
 cudaError_t launch_col_bits(const bsm_mat *X, uint32_t *bits, cudaStream_t s);
 cudaError_t launch_blk_rows(const bsm_mat *X, int32_t *rows, cudaStream_t s);

@@ -260,16 +260,12 @@ __device__ __forceinline__ int32_t col_rank(const uint32_t *bm, const int32_t *w
     return wpre[j >> 5] + __popc(w & ((1u << (j & 31)) - 1u));
 }
 
-__global__ void __launch_bounds__(kThreads) k_sym_fill(SymbolicArgs a, const uint32_t *bitmaps,
-                                                       FillOut o) {
-    extern __shared__ uint32_t smem[];
-    __shared__ int32_t wtmp[32];
-    if (a.status && *a.status != 0) return;
+__device__ __forceinline__ void sym_fill_row(const SymbolicArgs &a, const uint32_t *bitmaps, const FillOut &o, int i,
+                                             uint32_t *smem, int32_t *wtmp) {
     const int nw = a.nwords;
     uint32_t *bm = smem;
     int32_t *wpre = reinterpret_cast<int32_t *>(smem + nw);
     int32_t *cnt = wpre + nw;
-    const int i = o.row0 + blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t crow = o.crow_ptr[i];
     const int32_t ccnt = (int32_t)(o.crow_ptr[i + 1] - crow);
@@ -377,6 +373,18 @@ __global__ void __launch_bounds__(kThreads) k_sym_fill(SymbolicArgs a, const uin
     }
 }
 
+__global__ void __launch_bounds__(kThreads) k_sym_fill(SymbolicArgs a, const uint32_t *bitmaps, FillOut o,
+                                                       int32_t nrows) {
+    extern __shared__ uint32_t smem[];
+    __shared__ int32_t wtmp[32];
+    if (a.status && *a.status != 0) return;
+    if (a.stale && (*a.stale != 0) != (a.when_stale != 0)) return;
+    for (int r = blockIdx.x; r < nrows; r += gridDim.x) {
+        sym_fill_row(a, bitmaps, o, o.row0 + r, smem, wtmp);
+        __syncthreads();
+    }
+}
+
 // smallest norm (0 where one is NaN): every product of norms then exceeds a
 // threshold that the product of the two smallest exceeds, since rounding is
 // monotone
@@ -404,6 +412,18 @@ __global__ void k_col_bits(int32_t nbr, const int64_t *row_ptr, const int32_t *c
             atomicOr(&bits[(int64_t)col_idx[b] * words + (i >> 5)], 1u << (i & 31));
 }
 
+// one warp per block column: every entry of the copy, a permutation of the blocks, in its place?
+__global__ void k_check_columns(int32_t nbc, const int64_t *t_ptr, const int32_t *t_row, const int32_t *t_blk,
+                                const int64_t *row_ptr, const int32_t *col_idx, int32_t *stale) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < nbc; j += nwarp)
+        for (int64_t e = t_ptr[j] + lane; e < t_ptr[j + 1]; e += 32) {
+            const int32_t i = t_row[e], b = t_blk[e];
+            if (col_idx[b] != j || b < row_ptr[i] || b >= row_ptr[i + 1]) *stale = 1;
+        }
+}
+
 // Fill through B's columns.  Same outputs as k_sym_fill, but every C block
 // (i, j) is built from B's column j (B transposed: ascending k), so its
 // products come out in ascending k already and are written contiguously
@@ -429,6 +449,7 @@ __global__ void __launch_bounds__(kThreads) k_sym_fill_cols(SymbolicArgs a, cons
     __shared__ unsigned long long a_min;
     __shared__ int32_t wtmp[32];
     if (a.status && *a.status != 0) return;
+    if (a.stale && (*a.stale != 0) != (a.when_stale != 0)) return;
     const int nw = a.nwords;
     uint32_t *bm = smem;
     int32_t *wpre = reinterpret_cast<int32_t *>(smem + nw);
@@ -974,6 +995,14 @@ cudaError_t launch_col_bits(const bsm_mat *X, uint32_t *bits, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+cudaError_t launch_check_columns(const bsm_mat *X, int32_t *stale, cudaStream_t s) {
+    if (X->nnzb == 0) return cudaSuccess;
+    k_check_columns<<<grid_for((int64_t)X->nbc * 32), kThreads, 0, s>>>(X->nbc, X->t_ptr, X->t_row, X->t_blk, X->row_ptr,
+                                                                        X->col_idx, stale);
+    count_launch(1);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_symbolic_fill_cols(const SymbolicArgs &a, const uint32_t *bitmaps, const FillOut &o,
                                       const int64_t *bt_ptr, const int32_t *bt_k, const int32_t *bt_b,
                                       const uint32_t *bt_bits, cudaStream_t s, int32_t nrows) {
@@ -999,7 +1028,8 @@ cudaError_t launch_symbolic_fill(const SymbolicArgs &a, const uint32_t *bitmaps,
     if (nrows <= 0) return cudaSuccess;
     const int smem = (int)symbolic_fill_smem_bytes(a.nwords, o.max_ccnt, o.nchunk);
     if (const cudaError_t e = allow_dynamic_smem(k_sym_fill, smem)) return e;
-    k_sym_fill<<<nrows, kThreads, smem, s>>>(a, bitmaps, o);
+    // with a.stale most often nothing to do: few CTAs that end at once
+    k_sym_fill<<<a.stale ? std::min(nrows, 152) : nrows, kThreads, smem, s>>>(a, bitmaps, o, nrows);
     count_launch(1);
     return cudaGetLastError();
 }
