@@ -1756,6 +1756,19 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
             n_marked = C->n_marked;
             groups = C->item_groups;
             uses_cores = pl.uses_cores;
+            // the recomputed pattern may hold blocks of other shapes at the eager call's positions
+            if (order && (n_marked || groups) && (use_filter || A->plan.kind != 0 || B->plan.kind != 0)) {
+                Regroup rg{};
+                rg.n = nitems; rg.order = order; rg.n_lane = n_marked; rg.groups = groups; rg.blk_rc = c_rc;
+                rg.by_cols = rprec == BSM_P_OZAKI; rg.lane_6x6 = !needs_plain(kprec); rg.status = C->status;
+                if ((sst = sc.get(&rg.new_order, (size_t)nitems)) || (sst = sc.get(&rg.new_n_lane, 1)) ||
+                    (sst = sc.get(&rg.new_groups, kSplitGroups - 1)) || (sst = sc.get(&rg.counts, kRegroupWords)) ||
+                    (sst = cuda_check(launch_regroup(rg, g_stream), "order of the blocks")))
+                    return sst;
+                order = rg.new_order;
+                if (n_marked) n_marked = rg.new_n_lane;
+                if (groups) groups = rg.new_groups;
+            }
         } else if (whole) {
             if ((sst = ensure_row_rank(A))) return sst;
             const int32_t tile = tune_of(rprec)[BSM_TUNE_SCHED_TILE];

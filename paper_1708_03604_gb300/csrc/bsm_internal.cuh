@@ -287,8 +287,26 @@ __host__ __device__ constexpr bool half_rows(int rows) { return ((rows - 1) & 15
 // some output block ends in half a tile row; some has a whole one; some product
 // ends in half a k-step
 constexpr int kHalfRows = 1, kWholeRows = 2, kHalfInner = 4;
-inline int split_group(int rows) { return rows > 24 ? 0 : rows > 16 ? 1 : rows > 8 ? 2 : 3; }
+__host__ __device__ constexpr int split_group(int rows) { return rows > 24 ? 0 : rows > 16 ? 1 : rows > 8 ? 2 : 3; }
 constexpr int kWorkCounters = kSplitGroups + 1;  // tickets of the groups and of the lane items
+
+// The order of an eager call's blocks (its groups and its lane items, either may be
+// null) for a pattern of the same numbers whose blocks may have other shapes: copied
+// where every position holds a block of its class, else the blocks class by class.
+struct Regroup {
+    int64_t n;
+    const int32_t *order;
+    const int64_t *n_lane, *groups;
+    const int32_t *blk_rc;
+    int32_t by_cols;            // groups of one tile column (Ozaki path), else by height
+    int32_t lane_6x6;           // the lane kernels take 6 x 6 blocks
+    const int32_t *status;
+    int32_t *new_order;         // [n]
+    int64_t *new_n_lane, *new_groups;  // [1], [kSplitGroups - 1]
+    unsigned long long *counts;        // [kRegroupWords]
+};
+constexpr int kRegroupWords = 2 * (kSplitGroups + 1) + 1;
+cudaError_t launch_regroup(const Regroup &r, cudaStream_t s);
 
 // ---------------------------------------------------------------- numeric
 struct NumericArgs {

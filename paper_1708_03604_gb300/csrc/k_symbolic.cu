@@ -885,6 +885,57 @@ __global__ void k_class_keys(int64_t n, const int32_t *blk_rc, const int32_t *si
     }
 }
 
+// the class of the block at `pos` of the eager order and the one it belongs in: a
+// group, or kSplitGroups for the lane items
+struct BlockClass { int here, own; };
+__device__ __forceinline__ BlockClass block_class(const Regroup &r, int64_t pos) {
+    const int32_t rc = r.blk_rc[r.order[pos] & 0x7fffffff];
+    const int m = rc_rows(rc), n = rc_cols(rc);
+    const int own = !r.groups ? 0 : r.by_cols ? n <= 8 : split_group(m);
+    if (r.n_lane && pos >= r.n - *r.n_lane)
+        return {kSplitGroups, m * n <= 16 || (m == 5 && n == 5) || (r.lane_6x6 && m == 6 && n == 6) ? kSplitGroups : own};
+    int here = 0;
+    for (int g = 0; g < kSplitGroups - 1 && r.groups; ++g) here += pos >= r.groups[g];
+    return {here, own};
+}
+
+// counts[c] = blocks of class c, counts[kSplitGroups + 1] = blocks out of their class
+__global__ void __launch_bounds__(kThreads) k_regroup_count(Regroup r) {
+    if (r.status && *r.status != 0) return;
+    const int lane = threadIdx.x & 31;
+    unsigned long long mine[kSplitGroups + 2] = {};
+    for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~int64_t(31); base < r.n;
+         base += (int64_t)gridDim.x * blockDim.x) {
+        const BlockClass c = base + lane < r.n ? block_class(r, base + lane) : BlockClass{-1, -1};
+#pragma unroll
+        for (int g = 0; g <= kSplitGroups; ++g) mine[g] += __popc(__ballot_sync(0xffffffffu, c.own == g));
+        mine[kSplitGroups + 1] += __popc(__ballot_sync(0xffffffffu, c.own != c.here));
+    }
+#pragma unroll
+    for (int g = 0; g < kSplitGroups + 2; ++g)
+        if (lane == 0 && mine[g]) atomicAdd(&r.counts[g], mine[g]);
+}
+
+__global__ void __launch_bounds__(kThreads) k_regroup_place(Regroup r) {
+    if (r.status && *r.status != 0) return;
+    const bool same = r.counts[kSplitGroups + 1] == 0;
+    unsigned long long *taken = r.counts + kSplitGroups + 2;
+    for (int64_t pos = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; pos < r.n; pos += (int64_t)gridDim.x * blockDim.x) {
+        int64_t to = pos;
+        if (!same) {
+            const int own = block_class(r, pos).own;
+            to = (int64_t)atomicAdd(&taken[own], 1ull);
+            for (int g = 0; g < own; ++g) to += (int64_t)r.counts[g];
+        }
+        r.new_order[to] = r.order[pos];
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *r.new_n_lane = (int64_t)r.counts[kSplitGroups];
+        int64_t end = 0;
+        for (int g = 0; g < kSplitGroups - 1; ++g) r.new_groups[g] = end += (int64_t)r.counts[g];
+    }
+}
+
 // lower bounds of thresholds in sorted keys (one thread each)
 struct GroupThr { uint32_t v[kSplitGroups - 1]; };
 __global__ void k_group_bounds(const uint32_t *keys, int64_t n, GroupThr t, int64_t *out) {
@@ -910,6 +961,16 @@ inline int grid_for(int64_t n, int threads = kThreads) {
 }  // namespace
 
 // =================================================================== launchers
+cudaError_t launch_regroup(const Regroup &r, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(r.counts, 0, kRegroupWords * sizeof(unsigned long long), s);
+    if (e != cudaSuccess) return e;
+    const int grid = std::min(grid_for(r.n), 152 * 8);
+    k_regroup_count<<<grid, kThreads, 0, s>>>(r);
+    k_regroup_place<<<grid, kThreads, 0, s>>>(r);
+    count_launch(2);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_group_bounds(const uint32_t *keys, int64_t n, const uint32_t (&thr)[kSplitGroups - 1],
                                 int64_t *out, cudaStream_t s) {
     GroupThr t;

@@ -1,6 +1,7 @@
 """No-sync calls whose recomputed pattern has the eager call's sizes but other
 blocks in the same places (GPU): new values move the filter's decisions from one
-block to another.  The column copy of B comes from an earlier pattern of it; the
+block to another.  The order, groups and variant marks of the numeric kernels
+come from the eager call, the column copy of B from an earlier pattern of it; the
 result must be the new pattern's, against the oracle."""
 import numpy as np
 import pytest
@@ -9,6 +10,8 @@ from paper_1708_03604_gb300 import inputs as I
 from tests.helpers import random_bcsr, rel_fro
 
 pytestmark = pytest.mark.gpu
+
+TOL = {"fp64": 1e-12, "fp64_dmma": 1e-12, "tf32x3": 1e-6, "bf16x6": 1e-6, "bf16x3": 1e-4, "ozaki": 1e-13}
 
 
 @pytest.fixture(scope="module")
@@ -29,6 +32,39 @@ def _block_values(X, seed, on):
     rng = np.random.default_rng(seed)
     Y.data[:] = rng.uniform(0.5, 1.5, len(X.data)) * rng.choice([-1.0, 1.0], len(X.data)) * scale
     return Y
+
+
+def _full(rows, cols):
+    r, c = np.divmod(np.arange(len(rows) * len(cols)), len(cols))
+    return I.assemble(rows, cols, r, c, None, seed=1)
+
+
+# heights of the block rows: every height class twice, and tiny blocks (3 columns) beside large ones
+@pytest.mark.parametrize("heights", [(5, 23, 40, 13), (8, 9), (17, 16, 32), (2, 23), (1, 4, 40)], ids=str)
+@pytest.mark.parametrize("prec", sorted(TOL))
+def test_blocks_of_other_shapes(bsm, oracle, prec, heights):
+    rows = np.array(heights * 2, np.int32)                 # rows i and i + n have one height
+    n = len(heights)
+    inner, cols = np.array([7, 16], np.int32), np.array([3, 6, 24], np.int32)
+    Ah, Bh = _full(rows, inner), random_bcsr(inner, cols, 1.0, seed=2)
+    # kept in the eager call: row q of the first or of the second n; then the other one
+    first = np.arange(n) % 2 == 0
+    keep = np.concatenate([first, ~first])
+    on = [np.repeat(k, len(inner)) for k in (keep, ~keep)]
+    A1, A2 = (_block_values(Ah, s, o) for s, o in zip((3, 4), on))
+    A, B = bsm.Matrix.from_host(A1), bsm.Matrix.from_host(Bh)
+    for flush in (0, 4):
+        C = bsm.multiply(1.5, A, B, eps=1e-3, prec=prec, flush_every=flush)
+        for X in (A2, A1):
+            A.set_data(X.data)
+            bsm.multiply(1.5, A, B, Cm=C, eps=1e-3, prec=prec, flush_every=flush, no_sync=True)
+            ref = oracle.multiply(1.5, X, Bh, eps=1e-3).C
+            assert bsm.bsm_get_status(C.h) == 0
+            rp, ci, _ = C.pattern()
+            np.testing.assert_array_equal(rp, ref.row_ptr)
+            np.testing.assert_array_equal(ci, ref.col_idx)
+            # (flush_every 4 of the two-piece paths: four products share an FP32 sum)
+            assert rel_fro(C.data_host(), ref.data) <= (TOL[prec] if flush == 0 else 2 * TOL[prec])
 
 
 # B = X + 0 by a filtered add: X holds two patterns, the second one block column further, and the values choose
