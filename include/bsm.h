@@ -420,11 +420,12 @@ bsm_status bsm_block_norms(bsm_t X, double *out);
  *   recomputed sizes differ, the device sets C's status word
  *   (bsm_get_status -> BSM_ERR_CAPACITY) and writes nothing into C.  Stacks
  *   are not rebuilt.
- *   B keeps a column-major copy of its pattern until that changes and, where
- *   its columns are long enough for them (on average a block per 32 block rows
- *   and 48 more, 4e6 products), a bitmap of every column: less than 4 bytes per
- *   block of B and at most 256 MB.  Where their memory is refused the multiply
- *   goes on without them.
+ *   B keeps a column-major copy of its pattern until that changes and, from
+ *   5e5 products on where its columns are long enough for them (on average 16
+ *   blocks and two per 96 block rows with a threshold, 56 and one per 32
+ *   without), a bitmap of every column: less than 6 bytes per block of B and at
+ *   most 256 MB.  Where their memory is refused the multiply goes on without
+ *   them.
  */
 bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C,
                         double filter_eps, const bsm_opts *opts);

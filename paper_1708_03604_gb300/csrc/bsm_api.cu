@@ -621,19 +621,27 @@ bsm_status ensure_transpose(bsm_mat *X) {
 
 // Whether the fill of `nprod` products goes through bitmaps of B's columns, a word
 // for every 32 inner blocks.  Per C block the bitmaps read two words and expand one
-// per word of the inner dimension, and the walk reads the column's blocks twice; the
-// bitmaps' set-up is worth some 48 blocks of the walk.  Fill phase in ms, walk and
-// bitmaps, by words and blocks per column, random and banded columns:
-//   32 words   64: 4.0 and 4.0, 0.92 and 1.14   96: 6.6 and 4.6, 1.88 and 1.89
-//   125        144: 9.2 and 10.3, 1.08 and 1.38   224: 16.3 and 11.4, 2.36 and 2.33
-//   375        320: 6.6 and 8.4, 0.74 and 0.91   448: 10.8 and 9.4, 1.38 and 1.28
-//   938        100: 20.1 and 113, 23.3 and 135   1000: 16.2 and 16.9, 2.34 and 1.98
-// Below 4e6 products the difference is under 0.1 ms, less than making them.  By the
-// rule they take less than 4 bytes per block of B; they stay on the handle while its
+// per word of the inner dimension; the walk reads the column's blocks twice, 32 at a
+// time, and with a threshold the norms of those that meet a block of A.  Times of the
+// walk over those of the bitmaps in the fill phase, random and banded columns, by
+// words and blocks per column:
+//   with a threshold      10   24: 1.21, 1.02   36: 1.74, 1.36   56: 2.02, 1.52
+//                         63   48: 1.05, 1.10   64: 1.14, 1.08  112: 2.08, 1.64
+//                        375  192: 0.77, 0.87  256: 0.97, 1.02  384: 1.38, 1.39
+//                        938  256: 0.40, 0.53  640: 0.99, 1.11  950: 1.46, 1.58
+//   without                4   48: 0.85, 0.83   80: 0.85, 0.85
+//                         16   64: 1.02, 0.89   80: 1.31, 1.10
+//                         63   80: 0.85, 0.86  112: 1.09, 0.96  160: 1.44, 1.12
+//                        375  320: 0.79, 0.82  448: 1.14, 1.08
+//                        938  100: 0.18, 0.17  900: 0.89, 1.07
+// Below 5e5 products the difference is less than what making them costs.  By the rule
+// they take less than 6 bytes per block of B; they stay on the handle while its
 // pattern does, up to 256 MB.
-bool fill_bitmaps(const bsm_mat *B, int64_t nprod, int32_t nwords, int64_t max_ccnt) {
-    const int64_t words = ((int64_t)B->nbr + 31) / 32 * B->nbc;
-    return nprod >= (int64_t(1) << 22) && B->nnzb >= words + 48 * (int64_t)B->nbc && words <= (int64_t(1) << 26) &&
+bool fill_bitmaps(const bsm_mat *B, int64_t nprod, int32_t nwords, int64_t max_ccnt, bool filter) {
+    const int64_t column = ((int64_t)B->nbr + 31) / 32, words = column * B->nbc;
+    const bool longer = filter ? 3 * B->nnzb >= 2 * words + 48 * (int64_t)B->nbc
+                               : B->nnzb >= std::max<int64_t>(column + 56, 80) * B->nbc;
+    return longer && nprod >= (int64_t(1) << 19) && words <= (int64_t(1) << 26) &&
            symbolic_fill_cols_smem_bytes(nwords, (int32_t)max_ccnt, B->nbr, true) <= 200 * 1024;
 }
 
@@ -1582,7 +1590,7 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
             if ((st = cuda_check(launch_check_columns(B, stale, g_stream), "column copy"))) return st;
             sa.stale = stale;
         }
-        if (fill_bitmaps(B, nprod, nwords, max_ccnt)) {
+        if (fill_bitmaps(B, nprod, nwords, max_ccnt, use_filter)) {
             if (!no_sync && (st = ensure_col_bits(B))) return st;
             col_bits = B->t_bits;
         }

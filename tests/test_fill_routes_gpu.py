@@ -57,7 +57,7 @@ def _bitmap_bytes(B):
 
 
 # around a word and around the 32 words a warp expands at a time; C of 650 x 645 blocks
-@pytest.mark.parametrize("nbk", [64, 65, 95, 1023, 1024, 1025])
+@pytest.mark.parametrize("nbk", [65, 95, 96, 1023, 1024, 1025])
 @pytest.mark.parametrize("eps", [0.0, 1e-9, 1.0])
 def test_bitmaps(bsm, oracle, nbk, eps):
     rows, cols = I.uniform_sizes(650, 1), I.uniform_sizes(645, 2)
@@ -65,7 +65,7 @@ def test_bitmaps(bsm, oracle, nbk, eps):
     occ = 0.9 if nbk < 100 else 0.12
     Ah, Bh = random_bcsr(rows, inner, occ, seed=91), random_bcsr(inner, cols, occ, seed=92)
     asked = _check(bsm, oracle, Ah, Bh, eps)
-    if eps < 1.0:        # 4.2e6 products or more, columns of 48 blocks more than their words
+    if eps == 1e-9 or (eps == 0.0 and nbk > 1000):   # long enough columns with a threshold, without one
         assert _bitmap_bytes(Bh) in asked
 
 
@@ -77,18 +77,19 @@ def _columns(nbk, nbc, length, seed):
                       seed=seed)
 
 
-@pytest.mark.parametrize("length,bitmaps", [(85, False), (86, True)])
-def test_short_columns_are_walked(bsm, oracle, length, bitmaps):
-    """1,200 inner blocks are 38 words a column, 86 with 48 more."""
+@pytest.mark.parametrize("eps,length,bitmaps", [(0.0, 93, False), (0.0, 94, True), (1e-9, 41, False), (1e-9, 42, True)])
+def test_short_columns_are_walked(bsm, oracle, eps, length, bitmaps):
+    """1,200 inner blocks are 38 words a column: 56 blocks more without a threshold, two thirds and 16 with one."""
     Ah, Bh = random_bcsr(I.uniform_sizes(1100, 1), I.uniform_sizes(1200, 1), 0.07, seed=93), _columns(1200, 1000, length, 94)
-    for eps in (0.0, 1e-9):
-        assert (_bitmap_bytes(Bh) in _check(bsm, oracle, Ah, Bh, eps)) == bitmaps
+    assert (_bitmap_bytes(Bh) in _check(bsm, oracle, Ah, Bh, eps)) == bitmaps
 
 
-def test_few_products_are_walked(bsm, oracle):
-    bs = I.uniform_sizes(200, 1)
-    Ah, Bh = random_bcsr(bs, I.uniform_sizes(70, 1), 0.5, seed=95), random_bcsr(I.uniform_sizes(70, 1), bs, 0.5, seed=96)
-    assert _bitmap_bytes(Bh) not in _check(bsm, oracle, Ah, Bh, 0.0)
+@pytest.mark.parametrize("rows,bitmaps", [(81, False), (140, True)])
+def test_few_products_are_walked(bsm, oracle, rows, bitmaps):
+    """Columns of 66 blocks on average, 4.2e5 and 1.2e6 products."""
+    bs, cs, inner = I.uniform_sizes(rows, 1), I.uniform_sizes(rows + 2, 1), I.uniform_sizes(70, 1)
+    Ah, Bh = random_bcsr(bs, inner, 0.95, seed=95), random_bcsr(inner, cs, 0.95, seed=96)
+    assert (_bitmap_bytes(Bh) in _check(bsm, oracle, Ah, Bh, 1e-9)) == bitmaps
 
 
 def test_refused_bitmaps_fall_back_to_the_walk(bsm, oracle):

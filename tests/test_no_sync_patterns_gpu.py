@@ -68,7 +68,7 @@ def test_blocks_of_other_shapes(bsm, oracle, prec, heights):
 
 
 # B = X + 0 by a filtered add: X holds two patterns, the second one block column further, and the values choose
-@pytest.mark.parametrize("rows,inner,cols,occ", [(9, 40, 37, 0.1), (300, 200, 300, 0.3)], ids=["walk", "bitmaps"])
+@pytest.mark.parametrize("rows,inner,cols,occ", [(9, 40, 37, 0.1), (300, 200, 300, 0.3)], ids=["walk", "bitmaps_with_eps"])
 @pytest.mark.parametrize("eps", [0.0, 1e-9])
 def test_pattern_of_b(bsm, oracle, rows, inner, cols, occ, eps):
     one = random_bcsr(I.uniform_sizes(inner, 2), I.uniform_sizes(cols, 1), occ, seed=11)
@@ -91,7 +91,7 @@ def test_pattern_of_b(bsm, oracle, rows, inner, cols, occ, eps):
     A, X, Ym = bsm.Matrix.from_host(Ah), bsm.Matrix.from_host(X1), bsm.Matrix.from_host(Y)
     Z = bsm.add(1.0, X, 1.0, Ym, eps=1e-3)
     C = bsm.multiply(1.0, A, Z, eps=eps)
-    assert (C.counts().products >= 1 << 22) == (rows == 300)
+    assert (C.counts().products >= 1 << 19) == (rows == 300)
     for v, ref in ((X1, refs[0]), (X2, refs[1]), (X1, refs[0]), (X2, refs[1])):
         X.set_data(v.data)
         bsm.add(1.0, X, 1.0, Ym, Z=Z, eps=1e-3, no_sync=True)
