@@ -20,10 +20,10 @@ LIB = os.path.join(PKG, "libbsm.so")
 BUILD_DEBUG = os.path.join(PKG, "_build_debug")
 LIB_DEBUG = os.path.join(PKG, "libbsm_debug.so")
 SOURCES = ["bsm_api.cu", "k_symbolic.cu", "k_numeric.cu", "k_split_tf32x3.cu", "k_split_bf16x3.cu",
-           "k_split_bf16x6.cu", "k_group.cu", "k_tile.cu", "k_add.cu", "k_panel.cu",
+           "k_split_bf16x6.cu", "k_group.cu", "k_tile.cu", "k_warp.cu", "k_add.cu", "k_panel.cu",
            "bsm_static.cu", "k_probe.cu"]
 HEADERS = [os.path.join(CSRC, "bsm_internal.cuh"), os.path.join(CSRC, "numeric_debug.cuh"),
-           os.path.join(CSRC, "numeric_split.cuh"),
+           os.path.join(CSRC, "numeric_split.cuh"), os.path.join(CSRC, "numeric_warp.cuh"),
            os.path.join(CSRC, "numeric_items.cuh"), os.path.join(ROOT, "include", "bsm.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",

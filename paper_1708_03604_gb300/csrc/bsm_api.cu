@@ -174,6 +174,17 @@ bool mixed_sizes(const std::vector<int32_t> &v) {
     return std::any_of(v.begin(), v.end(), [&](int32_t x) { return x != v[0]; });
 }
 
+int32_t distinct_sizes(const std::vector<int32_t> &v) {
+    bool seen[kMaxBlockDim + 1] = {};
+    int32_t n = 0;
+    for (int32_t x : v)
+        if (!seen[x]) {
+            seen[x] = true;
+            ++n;
+        }
+    return n;
+}
+
 bool same_vec(const std::vector<int32_t> &a, const std::vector<int32_t> &b) { return a == b; }
 
 // Phase marks of a multiply: CUDA events on the library stream when
@@ -1751,6 +1762,7 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
         na.flush_every = opts.flush_every;
         na.max_out_rows = A->max_bs_row; na.max_out_cols = B->max_bs_col;
         na.mixed_k = mixed_sizes(A->h_col_bs);
+        na.out_shapes = distinct_sizes(A->h_row_bs) * distinct_sizes(B->h_col_bs);
         if (A->dtype != BSM_FP64) na.each_product = no_sync ? pl.each_product : each_product_of(rprec);
         na.x_pack = pkA.words; na.x_pack_off = pkA.off;
         na.y_pack = pkB.words; na.y_pack_off = pkB.off;
@@ -2048,6 +2060,7 @@ bsm_status bsm_multiply_backward(double alpha, bsm_t C, const void *dC_data, bsm
         na.prec = kprec;
         na.max_out_rows = OUT->max_bs_row; na.max_out_cols = OUT->max_bs_col;
         na.mixed_k = mixed_sizes(side == 0 ? B->h_col_bs : A->h_row_bs);
+        na.out_shapes = distinct_sizes(OUT->h_row_bs) * distinct_sizes(OUT->h_col_bs);
         if (C->dtype != BSM_FP64) na.each_product = each_product_of(opts.prec);
         na.flush_every = opts.flush_every;
         na.x_pack = pkX.words; na.x_pack_off = pkX.off;

@@ -327,7 +327,6 @@ struct NumericArgs {
     int32_t dtype;
     int32_t prec;
     int32_t flush_every;
-    EachProduct each_product;   // FP32 data
     // pre-split operand planes (tensor-core paths)
     const void *x_pack; const int64_t *x_pack_off;
     const void *y_pack; const int64_t *y_pack_off;
@@ -362,6 +361,10 @@ struct NumericArgs {
     int64_t x_len, y_len;       // operand elements
     int64_t out_len, old_len;   // output elements, old output elements (beta != 0)
     int64_t x_pack_words, y_pack_words;  // packed planes (0: none)
+    // CUDA-core kernels (last: among the fields above, 300 block rows of 1 to 40 took
+    // 2.95 ms for 2.89 in BF16x6)
+    EachProduct each_product;   // FP32 data
+    int32_t out_shapes;         // shapes that the output's block sizes can form
 };
 // Debug builds (BSM_DEBUG): bits of the bounds checks of the last numeric
 // launch (read and cleared; 0 in release builds).
@@ -383,6 +386,9 @@ cudaError_t launch_numeric_tile(const NumericArgs &a, cudaStream_t s, int *grid)
 cudaError_t launch_split_tf32x3(const NumericArgs &a, cudaStream_t s, int threads, int *grid);
 cudaError_t launch_split_bf16x3(const NumericArgs &a, cudaStream_t s, int threads, int *grid);
 cudaError_t launch_split_bf16x6(const NumericArgs &a, cudaStream_t s, int threads, int *grid);
+// few output blocks, either data (k_warp.cu)
+cudaError_t launch_numeric_warp(const NumericArgs &a, bool wide, cudaStream_t s, int *grid);
+uint32_t warp_debug_bits(cudaStream_t s);
 uint32_t split_tf32x3_debug_bits(cudaStream_t s);
 uint32_t split_bf16x3_debug_bits(cudaStream_t s);
 uint32_t split_bf16x6_debug_bits(cudaStream_t s);

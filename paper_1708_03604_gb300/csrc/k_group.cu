@@ -350,7 +350,8 @@ k_numeric_group(NumericArgs a) {
     constexpr uint32_t MASK = q_mask<BUILD>();
     if (a.status && *a.status != 0) return;
     const int lane = threadIdx.x & 31;
-    // a few blocks for each warp of the grid: a warp per block, so that all work
+    // a few blocks for each warp of the grid (tiny blocks; others are few_blocks then):
+    // a warp per block, so that all work
     const bool spread = a.n_items <= 4 * (int64_t)gridDim.x * (kGroupThreads / 32);
     __shared__ Window windows[kGroupThreads / 32];
     ItemRun run{&windows[threadIdx.x >> 5], 0, 0, a.n_items};

@@ -27,6 +27,7 @@
 #include "bsm_internal.cuh"
 #include "numeric_debug.cuh"
 #include "numeric_split.cuh"
+#include "numeric_warp.cuh"
 
 namespace bsm {
 
@@ -34,79 +35,11 @@ namespace {
 
 // =====================================================================
 // FP64 FMA on the CUDA cores, a warp or a lane per output block: the small
-// blocks of the FP64 tensor-core and Ozaki paths (BSM_P_FP64 has k_group.cu,
-// FP32 data k_tile.cu)
+// blocks of the FP64 tensor-core and Ozaki paths (BSM_P_FP64 has k_group.cu and,
+// for few blocks, k_warp.cu, FP32 data k_tile.cu)
 // =====================================================================
-template <int Q>
-__device__ __forceinline__ void cc_item(const NumericArgs &a, int64_t q, int lane) {
-    const double *__restrict__ X = static_cast<const double *>(a.x_data);
-    const double *__restrict__ Y = static_cast<const double *>(a.y_data);
-    double *__restrict__ O = static_cast<double *>(a.out_data);
-    const int32_t orc = a.out_blk_rc[q];
-    const int R = rc_rows(orc), S = rc_cols(orc);
-    const int RS = R * S;
-    const int64_t out_off = a.out_blk_off[q];
-    const int64_t p0 = a.seg_ptr[q], p1 = a.seg_ptr[q + 1];
-    const int64_t old = (a.beta != 0.0 && a.old_off) ? a.old_off[q] : -1;
-    const double *OLD = static_cast<const double *>(a.old_data);
-
-    for (int e0 = 0; e0 < RS; e0 += 32 * Q) {
-        int rr[Q], ss[Q];
-        double acc[Q];
-#pragma unroll
-        for (int u = 0; u < Q; ++u) {
-            const int e = e0 + lane + 32 * u;
-            const bool v = e < RS;
-            rr[u] = v ? e / S : 0;
-            ss[u] = v ? e % S : 0;
-            acc[u] = 0.0;
-        }
-        for (int64_t p = p0; p < p1; ++p) {
-            const int32_t ix = a.px[p], iy = a.py[p];
-            const double *xb = X + a.x_blk_off[ix];
-            const double *yb = Y + a.y_blk_off[iy];
-            const int32_t xrc = a.x_blk_rc[ix];
-            const int Tn = a.x_trans ? rc_rows(xrc) : rc_cols(xrc);
-            const int xs_r = a.x_trans ? 1 : Tn, xs_t = a.x_trans ? R : 1;
-            const int ys_t = a.y_trans ? 1 : S, ys_s = a.y_trans ? Tn : 1;
-            int xo[Q], yo[Q];
-#pragma unroll
-            for (int u = 0; u < Q; ++u) {
-                xo[u] = rr[u] * xs_r;
-                yo[u] = ss[u] * ys_s;
-            }
-            for (int t = 0; t < Tn; ++t) {
-#pragma unroll
-                for (int u = 0; u < Q; ++u) {
-                    const double xv = __ldg(xb + xo[u] + t * xs_t);
-                    const double yv = __ldg(yb + t * ys_t + yo[u]);
-                    acc[u] = fma(xv, yv, acc[u]);
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < Q; ++u) {
-            const int e = e0 + lane + 32 * u;
-            if (e < RS) {
-                double v = acc[u];
-                v = a.alpha * v;
-                if (old >= 0) v = fma(a.beta, OLD[old + e], v);
-                O[out_off + e] = v;
-            }
-        }
-    }
-}
-
-// up to 9 elements per lane per pass, more passes over the products for larger blocks
 __device__ __forceinline__ void cc_dispatch(const NumericArgs &a, int64_t q, int lane) {
-    const int32_t orc = a.out_blk_rc[q];
-    const int need = (rc_rows(orc) * rc_cols(orc) + 31) >> 5;
-    if (need <= 1) cc_item<1>(a, q, lane);
-    else if (need <= 2) cc_item<2>(a, q, lane);
-    else if (need <= 3) cc_item<3>(a, q, lane);
-    else if (need <= 4) cc_item<4>(a, q, lane);
-    else if (need <= 6) cc_item<6>(a, q, lane);
-    else cc_item<9>(a, q, lane);
+    warp_block<double, false>(a, q, lane);
 }
 
 // Tiny output blocks (at most 16 elements): one lane owns a whole block, so a
@@ -1170,6 +1103,30 @@ int num_sms() {
     return n;
 }
 
+// Whether the output has too few blocks for lane groups and register tiles, which
+// share warps among blocks of one shape: then a warp per block (k_warp.cu).  Times of
+// a warp per block over those of the sharing kernel, uniform patterns, 0.7 to 40
+// products a block:
+//   FP64  5 x 5        5,000 blocks 0.87-0.93   20,000 0.74-1.07    78,000 1.31-1.34
+//         8 x 8        5,000 0.89-0.98          40,000 0.74-0.90   160,000 0.98-1.16
+//         13 x 13      5,000 0.92-0.97          20,000 0.87-1.02    78,000 1.05-1.09
+//         23 x 23      3,000 0.87-0.95          20,000 1.01-1.05
+//         32 x 32      1,500 0.84-1.09          10,000 1.08-1.12
+//         5/13/23      5,000 0.62-0.77          80,000 0.82-0.90   160,000 1.08-1.28
+//         2/6          5,000 0.83-0.96          40,000 0.70-0.76   160,000 1.51-2.00
+//   FP32  5 x 5        5,000 0.79-0.85          20,000 0.83-1.74
+//         13 x 13      3,000 0.90-1.24          10,000 1.15-1.38
+//         5/13         5,000 0.78-0.97          20,000 0.78-1.11
+//         23 x 23, 32 x 32 and more: 1.2 to 3 from 1,000 on
+static bool few_blocks(const NumericArgs &a) {
+    const int area = a.max_out_rows * a.max_out_cols;
+    int per_sm;
+    if (area <= 16) per_sm = 0;
+    else if (a.dtype == BSM_FP64) per_sm = a.out_shapes > 1 ? (area <= 64 ? 400 : 800) : area > 288 ? 32 : area % 32 == 0 ? 400 : 200;
+    else per_sm = a.out_shapes > 1 ? (area <= 576 ? 100 : 0) : area <= 64 ? 64 : 0;
+    return a.n_items <= (int64_t)per_sm * num_sms();
+}
+
 cudaError_t launch_numeric(const NumericArgs &args, cudaStream_t s, NumericLaunch *info) {
     NumericArgs a = args;
     a.unit_alpha = a.alpha == 1.0;
@@ -1210,24 +1167,23 @@ cudaError_t launch_numeric(const NumericArgs &args, cudaStream_t s, NumericLaunc
         li = NumericLaunch{BSM_K_FP64_MMA, -1, kThreadsNum, grid, a.pass_mt > 0 ? a.pass_mt : 3,
                            a.pass_nt > 0 ? a.pass_nt : 3};
     } else if (!tc) {
-        int build = -1;
-        if (a.dtype == BSM_FP64) {
-            // the build by the largest output block: narrow up to 288 elements and
-            // beyond the wide ladder's single pass (768), wide between, where its
-            // larger Q fill more lane slots; narrow and wide in ms (3e10 useful
-            // FLOP, 10% occupancy): 16 x 16 23.9 and 24.3, 17 x 17 27.4 and 25.6,
-            // 18 x 18 26.2 and 25.1, 20 x 20 25.0 and 25.1, 23 x 23 26.1 and 24.8,
-            // 24 x 24 24.0 and 24.2, 32 x 32 24.5 and 24.7.  The tuner may ask for
-            // either; the small build only ever runs when every output block has at
-            // most 16 elements
-            const int area = a.max_out_rows * a.max_out_cols;
-            build = (area > 0 && area <= 16) ? kCcSmall : (area <= 288 || area > 768) ? kCcNarrow : kCcWide;
-            if (a.fp64_build == 1 && build != kCcSmall) build = kCcNarrow;
-            if (a.fp64_build == 2 && build != kCcSmall) build = kCcWide;
-            e = launch_numeric_group(a, build, s, &grid);
-        } else {
-            e = launch_numeric_tile(a, s, &grid);
-        }
+        const int area = a.max_out_rows * a.max_out_cols;
+        const bool few = few_blocks(a);
+        // the build by the largest output block: narrow up to 288 elements and
+        // beyond the wide ladder's single pass (768), wide between, where its
+        // larger Q fill more lane slots; narrow and wide in ms (3e10 useful
+        // FLOP, 10% occupancy): 16 x 16 23.9 and 24.3, 17 x 17 27.4 and 25.6,
+        // 18 x 18 26.2 and 25.1, 20 x 20 25.0 and 25.1, 23 x 23 26.1 and 24.8,
+        // 24 x 24 24.0 and 24.2, 32 x 32 24.5 and 24.7.  The tuner may ask for
+        // either; the small build only ever runs when every output block has at
+        // most 16 elements
+        int build = area > 0 && area <= 16 ? kCcSmall : area <= 288 || area > 768 ? kCcNarrow : kCcWide;
+        if (a.fp64_build == 1 && build != kCcSmall) build = kCcNarrow;
+        if (a.fp64_build == 2 && build != kCcSmall) build = kCcWide;
+        if (few) e = launch_numeric_warp(a, build == kCcWide, s, &grid);
+        else if (a.dtype == BSM_FP64) e = launch_numeric_group(a, build, s, &grid);
+        else e = launch_numeric_tile(a, s, &grid);
+        if (a.dtype != BSM_FP64) build = -1;
         li = NumericLaunch{BSM_K_FP64_CORES, build, kThreadsNum, grid, 0, 0};
     } else {
         if (a.prec == BSM_P_TF32x3) e = launch_split_tf32x3(a, s, tc_threads, &grid);
@@ -1243,7 +1199,7 @@ cudaError_t launch_numeric(const NumericArgs &args, cudaStream_t s, NumericLaunc
 }
 
 uint32_t numeric_debug_bits(cudaStream_t s) {
-    return read_debug_bits(s) | group_debug_bits(s) | tile_debug_bits(s) | split_tf32x3_debug_bits(s) |
+    return read_debug_bits(s) | group_debug_bits(s) | tile_debug_bits(s) | warp_debug_bits(s) | split_tf32x3_debug_bits(s) |
            split_bf16x3_debug_bits(s) | split_bf16x6_debug_bits(s);
 }
 
