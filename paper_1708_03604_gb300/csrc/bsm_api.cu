@@ -480,6 +480,17 @@ bsm_status ensure_row_rank(bsm_mat *X) {
     return BSM_OK;
 }
 
+// Whether n output blocks of a split path run in an instance per height class, with
+// fewer registers and more warps each, or all in the any-height one: the classes are
+// launched one after the other, each with its own tail.  Classes and one instance,
+// TF32x3, ms: 5/13/23 with 8 products a block 10,000 blocks 0.075 and 0.044, 20,000
+// 0.093 and 0.087, 40,000 0.142 and 0.153, 100,000 0.327 and 0.405; 7/20/40 10,000
+// 0.249 and 0.198, 20,000 0.306 and 0.300, 40,000 0.568 and 0.595.  Where several
+// products share a sum the classes' accumulators are part of the result.
+bool split_classes(int64_t n, int32_t flush_every) {
+    return std::abs(flush_every) > 1 || n > 128 * (int64_t)num_sms();
+}
+
 // Processing order of n output blocks for the numeric kernels: grouped by
 // block shape, larger blocks first, so that neighbouring warps run the same
 // code path and the heaviest items start early.
@@ -1736,9 +1747,11 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
     // one numeric pass over the output blocks [cb0, cb0 + nitems) holding nprod_pass
     // products (the whole C, or one row panel of a chunked multiply)
     float *plain_x = nullptr, *plain_y = nullptr;
-    // split paths: blocks of one tile row in their own kernel instance, unless
-    // the tuning fixes the pass rows; Ozaki path: blocks of one tile column
-    const bool want_groups = rprec == BSM_P_OZAKI || tune_of(rprec)[BSM_TUNE_PASS_MT] <= 0;
+    // split paths: a kernel instance per height class, unless the tuning fixes the
+    // pass rows; Ozaki path: blocks of one tile column
+    auto want_groups = [&](int64_t n) {
+        return rprec == BSM_P_OZAKI || (tune_of(rprec)[BSM_TUNE_PASS_MT] <= 0 && split_classes(n, opts.flush_every));
+    };
     // the CUDA-core kernels group small blocks by themselves: no variant marks in their order
     const bool cores = kprec == BSM_P_FP64 || (kprec == BSM_P_FP64_DMMA && A->dtype != BSM_FP64);
     const int order_prec = cores ? -1 : rprec;
@@ -1798,11 +1811,11 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
             rows_view.row_ptr = crow_ptr;
             if ((sst = shape_order(sc, nitems, c_rc + cb0, A->h_row_bs, B->h_col_bs, &order, &rows_view, A->row_rank,
                                    order_prec, &uses_cores, &n_marked, c_col + cb0, tile > 0 ? B->col_rank : nullptr, nbc,
-                                   tile > 0 ? tile : 0, want_groups ? &groups : nullptr)))
+                                   tile > 0 ? tile : 0, want_groups(nitems) ? &groups : nullptr)))
                 return sst;
         } else {  // a row panel: block-shape classes and variants only
             if ((sst = shape_order(sc, nitems, c_rc + cb0, A->h_row_bs, B->h_col_bs, &order, nullptr, nullptr, order_prec,
-                                   &uses_cores, &n_marked, nullptr, nullptr, 0, 0, want_groups ? &groups : nullptr)))
+                                   &uses_cores, &n_marked, nullptr, nullptr, 0, 0, want_groups(nitems) ? &groups : nullptr)))
                 return sst;
         }
         na.item_groups = groups;
@@ -2074,7 +2087,8 @@ bsm_status bsm_multiply_backward(double alpha, bsm_t C, const void *dC_data, bsm
         // one kernel instance per height class where it adds in the same order
         // (more block products per sum run two accumulators in some of them)
         const bool want_groups = is_tc(kprec) && kprec != BSM_P_OZAKI && std::abs(opts.flush_every) <= 1 &&
-                                 tune_of(opts.prec)[BSM_TUNE_PASS_MT] <= 0;
+                                 tune_of(opts.prec)[BSM_TUNE_PASS_MT] <= 0 &&
+                                 split_classes(OUT->nnzb, opts.flush_every);
         int64_t *groups = nullptr;
         if ((st = shape_order(sc, OUT->nnzb, OUT->blk_rc, OUT->h_row_bs, OUT->h_col_bs, &item_order, nullptr, nullptr,
                               kprec == BSM_P_FP64 || (kprec == BSM_P_FP64_DMMA && C->dtype != BSM_FP64) ? -1 : opts.prec,

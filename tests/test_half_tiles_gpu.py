@@ -50,22 +50,25 @@ def test_heights(bsm, oracle, prec, heights):
                 np.testing.assert_array_equal(c, got[-1])
 
 
-@pytest.mark.parametrize("flush", [4, -3])
+@pytest.mark.parametrize("flush", [0, 1, 4, -3])
 @pytest.mark.parametrize("prec", sorted(TOL))
-def test_several_products_a_sum(bsm, prec, flush):
-    """More than one block product a sum: the one-row instances add in two accumulators and the two-row ones in one,
-    so blocks of one tile row must be the bits of the any-height instance of one row, the others of that of two."""
+def test_classes(bsm, oracle, prec, flush):
+    """Enough blocks (22,500) for an instance per height class.  With more than one block product a sum the one-row
+    instances add in two accumulators and the two-row ones in one, so blocks of one tile row must be the bits of the
+    any-height instance of one row, the others of that of two; with one product a sum all three agree."""
     from paper_1708_03604_gb300 import autotune
-    rows = I.mixed_sizes(60, (5, 8, 9, 16, 17, 24, 25, 40), [1 / 8] * 8, seed=3)
-    mid, cols = I.mixed_sizes(60, (3, 8, 17), [1 / 3] * 3, seed=4), I.mixed_sizes(60, (6, 13, 24), [1 / 3] * 3, seed=5)
-    A = bsm.Matrix.from_host(random_bcsr(rows, mid, 0.3, seed=6))
-    B = bsm.Matrix.from_host(random_bcsr(mid, cols, 0.3, seed=7))
+    rows = I.mixed_sizes(150, (5, 8, 9, 16, 17, 24, 25, 40), [1 / 8] * 8, seed=3)
+    mid, cols = I.mixed_sizes(60, (3, 8, 17), [1 / 3] * 3, seed=4), I.mixed_sizes(150, (6, 13, 24), [1 / 3] * 3, seed=5)
+    Ah, Bh = random_bcsr(rows, mid, 0.4, seed=6), random_bcsr(mid, cols, 0.4, seed=7)
+    A, B = bsm.Matrix.from_host(Ah), bsm.Matrix.from_host(Bh)
     got = {}
     try:
         for pm in (-1, 2, 1):
             bsm.bsm_set_tuning(prec, "pass_mt", pm)
             C = bsm.multiply(1.0, A, B, prec=prec, flush_every=flush)
             got[pm] = C.data_host()
+            if pm == -1:
+                assert C.launch_config()["pass_mt"] == 0
     finally:
         autotune.reset(prec)
     rp, ci, _ = C.pattern()
@@ -73,3 +76,6 @@ def test_several_products_a_sum(bsm, prec, flush):
     low = np.repeat(m <= 16, m * n)
     np.testing.assert_array_equal(got[-1][low], got[1][low])
     np.testing.assert_array_equal(got[-1][~low], got[2][~low])
+    if flush in (0, 1):
+        np.testing.assert_array_equal(got[1], got[2])
+        assert rel_fro(got[-1], oracle.multiply(1.0, Ah, Bh).C.data) <= TOL[prec]
