@@ -349,17 +349,20 @@ bsm_status oz_lines(Scratch &sc, const bsm_mat *M, int role_y, int trans, OzLine
 struct Packed {
     int64_t *off = nullptr;  // [nnzb+1] word offsets
     uint32_t *words = nullptr;
+    bool whole = false;      // Ozaki path: in whole tiles and k-steps
+    int64_t *sizes = nullptr, *tmp = nullptr;
 };
 
-// Launch pack-size computation and its scan; the total lands in off[nnzb].
-bsm_status pack_prepare(Scratch &sc, const bsm_mat *M, int role_y, int trans, int prec, Packed &pk) {
-    int64_t *w = nullptr, *tmp = nullptr;
+// Launch pack-size computation and its scan; the total lands in off[nnzb].  `other`
+// (nullable, zeroed): the total in the other Ozaki layout.
+bsm_status pack_prepare(Scratch &sc, const bsm_mat *M, int role_y, int trans, int prec, Packed &pk,
+                        unsigned long long *other = nullptr) {
     bsm_status st;
-    if ((st = sc.get(&w, (size_t)M->nnzb)) != BSM_OK) return st;
-    if ((st = sc.get(&pk.off, (size_t)M->nnzb + 1)) != BSM_OK) return st;
-    if ((st = sc.get(&tmp, scan_tmp_elems(M->nnzb))) != BSM_OK) return st;
-    cudaError_t e = launch_pack_sizes(M, role_y, trans, prec, w, g_stream);
-    if (e == cudaSuccess) e = launch_scan_i64(w, pk.off, M->nnzb, tmp, g_stream);
+    if (!pk.off && ((st = sc.get(&pk.sizes, (size_t)M->nnzb)) || (st = sc.get(&pk.off, (size_t)M->nnzb + 1)) ||
+                    (st = sc.get(&pk.tmp, scan_tmp_elems(M->nnzb)))))
+        return st;
+    cudaError_t e = launch_pack_sizes(M, role_y, trans, prec, pk.whole, pk.sizes, other, g_stream);
+    if (e == cudaSuccess) e = launch_scan_i64(pk.sizes, pk.off, M->nnzb, pk.tmp, g_stream);
     return cuda_check(e, "pack sizes");
 }
 
@@ -368,7 +371,7 @@ bsm_status pack_fill(Scratch &sc, const bsm_mat *M, int role_y, int trans, int p
     bsm_status st;
     if ((st = sc.get(&pk.words, (size_t)total_words + 16)) != BSM_OK) return st;
     if (prec == BSM_P_OZAKI && (st = oz_lines(sc, M, role_y, trans, *ol))) return st;
-    return cuda_check(launch_pack(M, role_y, trans, prec, pk.off, pk.words, nullptr, g_stream,
+    return cuda_check(launch_pack(M, role_y, trans, prec, pk.whole, pk.off, pk.words, nullptr, g_stream,
                                   ol ? ol->line0 : nullptr, ol ? ol->exps : nullptr),
                       "pack");
 }
@@ -478,6 +481,20 @@ bsm_status ensure_row_rank(bsm_mat *X) {
     }
     X->row_rank = d;
     return BSM_OK;
+}
+
+// Whether the Ozaki operands are packed in whole tiles and k-steps.  Half tiles save
+// MMAs, but blocks that end in half a tile row after whole ones then run in two
+// kernels, each with a block's fixed costs, which few products do not pay.  Whole
+// over half, numeric pass and multiply, by products per block: 900 block rows of
+// 23 x 23 1.3: 0.91, 0.93   2.3: 0.94, 0.95   4.1: 0.98, 0.99; 320 rows 8: 1.07, 1.06;
+// 900 rows of 5/13/23 1.3: 0.89, 0.93   4: 0.92, 0.94   8: 0.99, 1.00   16: 1.07, 1.07.
+bool oz_whole_tiles(int64_t nprod, int64_t blocks, const std::vector<int32_t> &rows) {
+    return nprod < 5 * blocks && std::any_of(rows.begin(), rows.end(), [](int32_t r) { return r > 16 && half_rows(r); });
+}
+
+bool oz_few_blocks(const bsm_mat *A, const bsm_mat *B) {
+    return A->nbc > 0 && (int64_t)A->nbr * B->nbc <= 128 * (int64_t)num_sms();
 }
 
 // Whether n output blocks of a split path run in an instance per height class, with
@@ -1494,9 +1511,9 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
     if ((st = sc.get(&prod_cnt, nbr)) || (st = sc.get(&ccol_cnt, nbr)) || (st = sc.get(&celem_cnt, nbr)) ||
         (st = sc.get(&prod_ptr, (size_t)nbr + 1)) || (st = sc.get(&crow_ptr, (size_t)nbr + 1)) ||
         (st = sc.get(&celem_ptr, (size_t)nbr + 1)) || (st = sc.get(&stmp, scan_tmp_elems(nbr))) ||
-        (st = sc.get(&bitmaps, (size_t)nbr * nwords)) || (st = sc.get(&totals, 4)))
+        (st = sc.get(&bitmaps, (size_t)nbr * nwords)) || (st = sc.get(&totals, 6)))
         return st;
-    e = cudaMemsetAsync(totals, 0, 4 * sizeof(unsigned long long), g_stream);
+    e = cudaMemsetAsync(totals, 0, 6 * sizeof(unsigned long long), g_stream);
     if (e == cudaSuccess) e = launch_symbolic_count(sa, prod_cnt, ccol_cnt, celem_cnt, bitmaps, totals, g_stream);
     if (e == cudaSuccess) e = launch_scan_i64(prod_cnt, prod_ptr, nbr, stmp, g_stream);
     if (e == cudaSuccess) e = launch_scan_i64(ccol_cnt, crow_ptr, nbr, stmp, g_stream);
@@ -1506,8 +1523,13 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
     Packed pkA, pkB;
     const bool tc = is_tc(kprec);
     if (tc) {
-        if ((st = pack_prepare(sc, A, 0, 0, kprec, pkA))) return st;
-        if ((st = pack_prepare(sc, B, 1, 0, kprec, pkB))) return st;
+        // few blocks: by the products of a uniform pattern; else half, until the products are known
+        const bool oz = kprec == BSM_P_OZAKI;
+        if (oz)
+            pkA.whole = pkB.whole = no_sync ? pl.oz_whole : oz_few_blocks(A, B) && oz_whole_tiles(A->nnzb * B->nnzb / nbk,
+                                                                                                  (int64_t)nbr * nbc, A->h_row_bs);
+        if ((st = pack_prepare(sc, A, 0, 0, kprec, pkA, oz ? totals + 4 : nullptr))) return st;
+        if ((st = pack_prepare(sc, B, 1, 0, kprec, pkB, oz ? totals + 5 : nullptr))) return st;
     }
     int64_t nprod, nnzbC, lenC, nfilt, mnk, packA_words = 0, packB_words = 0, max_ccnt = 0;
     int nchunk = 8;
@@ -1533,14 +1555,15 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
         if ((st = cuda_check(launch_check_plan(pc, C->status, g_stream), "plan check"))) return st;
     } else {
         std::vector<int64_t> h_ccnt((size_t)nbr);
-        const int64_t *src[7] = {prod_ptr + nbr, crow_ptr + nbr, celem_ptr + nbr, (const int64_t *)totals,
+        const int64_t *src[9] = {prod_ptr + nbr, crow_ptr + nbr, celem_ptr + nbr, (const int64_t *)totals,
                                  (const int64_t *)(totals + 1), tc ? pkA.off + A->nnzb : nullptr,
-                                 tc ? pkB.off + B->nnzb : nullptr};
+                                 tc ? pkB.off + B->nnzb : nullptr, (const int64_t *)(totals + 4),
+                                 (const int64_t *)(totals + 5)};
         if (nbr > 0) {
             e = cudaMemcpyAsync(h_ccnt.data(), ccol_cnt, sizeof(int64_t) * nbr, cudaMemcpyDeviceToHost, g_stream);
             if ((st = cuda_check(e, "read counts"))) return st;
         }
-        if ((st = read_words(src, tc ? 7 : 5))) return st;
+        if ((st = read_words(src, kprec == BSM_P_OZAKI ? 9 : tc ? 7 : 5))) return st;
         nprod = g_host[0]; nnzbC = g_host[1]; lenC = g_host[2]; nfilt = g_host[3]; mnk = g_host[4];
         if (tc) {
             packA_words = g_host[5];
@@ -1571,6 +1594,14 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
                 panel_rows.push_back(r1);
                 r = r1;
             }
+        }
+        // the other layout: offsets again (0.02 ms; 7e4 products of 23 x 23 take 1 ms)
+        if (kprec == BSM_P_OZAKI && !oz_few_blocks(A, B) && nprod >= (int64_t(1) << 16) &&
+            oz_whole_tiles(nprod, nnzbC, A->h_row_bs)) {
+            packA_words = g_host[7];
+            packB_words = g_host[8];
+            pkA.whole = pkB.whole = true;
+            if ((st = pack_prepare(sc, A, 0, 0, kprec, pkA)) || (st = pack_prepare(sc, B, 1, 0, kprec, pkB))) return st;
         }
         while (nchunk > 1 && symbolic_fill_smem_bytes(nwords, (int32_t)max_ccnt, nchunk) > 160 * 1024) nchunk >>= 1;
         if (symbolic_fill_smem_bytes(nwords, (int32_t)max_ccnt, nchunk) > 220 * 1024)
@@ -1737,10 +1768,10 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
             return st;
         if (kprec == BSM_P_OZAKI && ((st = oz_lines(sc, A, 0, 0, olA)) || (st = oz_lines(sc, B, 1, 0, olB))))
             return st;
-        e = launch_pack(A, 0, 0, kprec, pkA.off, pkA.words, no_sync ? C->status : nullptr, g_stream, olA.line0,
+        e = launch_pack(A, 0, 0, kprec, pkA.whole, pkA.off, pkA.words, no_sync ? C->status : nullptr, g_stream, olA.line0,
                         olA.exps);
         if (e == cudaSuccess)
-            e = launch_pack(B, 1, 0, kprec, pkB.off, pkB.words, no_sync ? C->status : nullptr, g_stream,
+            e = launch_pack(B, 1, 0, kprec, pkB.whole, pkB.off, pkB.words, no_sync ? C->status : nullptr, g_stream,
                             olB.line0, olB.exps);
         if ((st = cuda_check(e, "pack"))) return st;
     }
@@ -1820,6 +1851,7 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
         }
         na.item_groups = groups;
         tile_masks(A->h_row_bs, A->h_col_bs, na);
+        if (pkA.whole) na.half_mask |= kAllWhole;
         na.n_lane_items = n_marked;
         if (needs_plain(kprec) && uses_cores && !plain_x) {  // unpacked pieces for the CUDA-core split variant
             const int np = split_pieces(rprec);
@@ -1923,6 +1955,7 @@ bsm_status bsm_multiply(double alpha, bsm_t A, bsm_t B, double beta, bsm_t C, do
         P.kind = 1; P.A = A; P.B = B; P.A_nnzb = A->nnzb; P.B_nnzb = B->nnzb; P.eps = filter_eps;
         P.prec = opts.prec; P.kprec = kprec; P.nprod = nprod; P.nnzb = nnzbC; P.len = lenC; P.max_ccnt = max_ccnt;
         P.uses_cores = uses_cores;
+        P.oz_whole = pkA.whole;
         if (A->dtype != BSM_FP64) P.each_product = each_product_of(rprec);
         P.nfilt = nfilt; P.mnk = mnk; P.nchunk = nchunk; P.packA = packA_words; P.packB = packB_words;
     }
@@ -2047,6 +2080,7 @@ bsm_status bsm_multiply_backward(double alpha, bsm_t C, const void *dC_data, bsm
         OzLines olX, olY;
         int64_t wx_words = 0, wy_words = 0;
         if (tc && nprod > 0) {
+            pkX.whole = pkY.whole = kprec == BSM_P_OZAKI && oz_whole_tiles(nprod, OUT->nnzb, OUT->h_row_bs);
             if ((st = pack_prepare(sc, X, 0, xt, kprec, pkX))) return st;
             if ((st = pack_prepare(sc, Y, 1, yt, kprec, pkY))) return st;
             const int64_t *src[2] = {pkX.off + X->nnzb, pkY.off + Y->nnzb};
@@ -2097,6 +2131,7 @@ bsm_status bsm_multiply_backward(double alpha, bsm_t C, const void *dC_data, bsm
         na.n_lane_items = n_marked;
         na.item_groups = groups;
         tile_masks(OUT->h_row_bs, side == 0 ? B->h_col_bs : A->h_row_bs, na);
+        if (pkX.whole) na.half_mask |= kAllWhole;
         if (needs_plain(kprec) && uses_cores && nprod > 0) {
             const int np = split_pieces(opts.prec);
             float *xp = nullptr, *yp = nullptr;

@@ -94,6 +94,7 @@ struct bsm_mat {
         int32_t nchunk = 1;
         int64_t packA = 0, packB = 0;
         bool uses_cores = false;  // some items run the CUDA-core split variant
+        bool oz_whole = false;    // Ozaki operands in whole tiles
         bsm::EachProduct each_product;
         int64_t u_nnzb = 0, u_len = 0;  // add: union before the norm filter
     } plan;
@@ -287,6 +288,7 @@ __host__ __device__ constexpr bool half_rows(int rows) { return ((rows - 1) & 15
 // some output block ends in half a tile row; some has a whole one; some product
 // ends in half a k-step
 constexpr int kHalfRows = 1, kWholeRows = 2, kHalfInner = 4;
+constexpr int kAllWhole = 8;  // operands packed in whole tiles and k-steps only
 __host__ __device__ constexpr int split_group(int rows) { return rows > 24 ? 0 : rows > 16 ? 1 : rows > 8 ? 2 : 3; }
 constexpr int kWorkCounters = kSplitGroups + 1;  // tickets of the groups and of the lane items
 
@@ -343,7 +345,7 @@ struct NumericArgs {
     // Ozaki path: two groups, the second of blocks of one tile column
     const int64_t *item_groups;
     int32_t group_mask;         // the groups that the output's block sizes can fill
-    int32_t half_mask;          // Ozaki path: kHalfRows | kWholeRows | kHalfInner
+    int32_t half_mask;          // Ozaki path: kHalfRows | kWholeRows | kHalfInner | kAllWhole
     int32_t group;              // set by the launcher: the group one launch covers
     const int32_t *status;      // nullable: the kernel does nothing when *status != 0
     unsigned long long *work_counter;  // kWorkCounters x 8 bytes of device memory, zeroed by the launcher
@@ -408,10 +410,12 @@ cudaError_t launch_oz_lines(const bsm_mat *M, int by_rows, int32_t *line0, int32
 struct PackInfo {
     int64_t total_words;        // 32-bit words
 };
-cudaError_t launch_pack_sizes(const bsm_mat *M, int role_y, int trans, int prec, int64_t *pack_words,
-                              cudaStream_t s);
+// whole: Ozaki operands in whole tiles and k-steps only; other (nullable): adds the
+// words of the other Ozaki layout
+cudaError_t launch_pack_sizes(const bsm_mat *M, int role_y, int trans, int prec, bool whole, int64_t *pack_words,
+                              unsigned long long *other, cudaStream_t s);
 // line0 / exps: the Ozaki path's line exponents of M in this role (else null)
-cudaError_t launch_pack(const bsm_mat *M, int role_y, int trans, int prec, const int64_t *pack_off,
+cudaError_t launch_pack(const bsm_mat *M, int role_y, int trans, int prec, bool whole, const int64_t *pack_off,
                         void *pack, const int32_t *status, cudaStream_t s, const int32_t *line0 = nullptr,
                         const int32_t *exps = nullptr);
 // Unpacked split pieces of M's data (split_pieces(prec) floats per element).

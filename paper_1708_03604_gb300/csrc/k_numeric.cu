@@ -335,6 +335,7 @@ template <bool HK> __host__ __device__ constexpr int oz_xstep(int R) {
     return 32 * ((HK ? kOzHW : kOzXW) * ((R - 1) / 16) +
                  (half_rows(R) ? (HK ? kOzQW : kOzHW) : (HK ? kOzHW : kOzXW)));
 }
+__host__ __device__ constexpr int oz_xstep_whole(int R) { return 32 * kOzXW * ((R + 15) / 16); }
 template <bool HK> __host__ __device__ constexpr int oz_ystep(int S) { return 32 * (HK ? kOzQW : kOzYW) * ((S + 7) / 8); }
 // ring words per lane per stage for passes of at most MAXN tiles (1 x MAXN)
 template <int MAXN>
@@ -421,7 +422,8 @@ __device__ __forceinline__ void oz_step(float (&acc)[kOzLevels][NTC][4], const u
 
 // One pass over a 1 x NTC super tile (16 x 8*NTC output elements) at (mt0, nt0),
 // staged through a ring laid out for passes of at most MAXN tiles.  HM: half a tile
-// of rows; HKS: some product has an HK step (the multiply's inner sizes tell).
+// of rows; HKS: some product has an HK step (the multiply's inner sizes tell); WT:
+// packs of whole tiles and k-steps.
 //
 // Bound by the latency of a warp's steps at eight warps an SM: 2,000 banded rows of
 // 23, the kernels of the half and of the whole tile rows, tensor pipe 42% and 48%
@@ -434,7 +436,7 @@ __device__ __forceinline__ void oz_step(float (&acc)[kOzLevels][NTC][4], const u
 // of 23 (1.96e7 products) 55.0 -> 47.5 ms, of blocks of 5 (8e7) 26.0 -> 19.8, of 13
 // (6.9e6) 7.34 -> 7.16, of 32 (4.6e5) 4.44 -> 4.13, the last two from the running
 // pointers and untested tiles alone.
-template <int NTC, int MAXN, bool HM, bool HKS>
+template <int NTC, int MAXN, bool HM, bool HKS, bool WT>
 __device__ __forceinline__ void oz_pass(const NumericArgs &a, int64_t q, int lane, int mt0, int nt0,
                                         uint32_t *ring) {
     constexpr int ST = kOzStages, SW = oz_sw<MAXN>();
@@ -443,7 +445,7 @@ __device__ __forceinline__ void oz_pass(const NumericArgs &a, int64_t q, int lan
     const int64_t p0 = a.seg_ptr[q], p1 = a.seg_ptr[q + 1];
     const uint32_t *XP = static_cast<const uint32_t *>(a.x_pack) + 4 * lane;
     const uint32_t *YP = static_cast<const uint32_t *>(a.y_pack) + 4 * lane;
-    const int xk = oz_xstep<false>(R), yk = oz_ystep<false>(S);
+    const int xk = WT ? oz_xstep_whole(R) : oz_xstep<false>(R), yk = oz_ystep<false>(S);
     constexpr int NV = HM ? 2 : 4;  // accumulator elements of a lane that count
     double *O = static_cast<double *>(a.out_data);
     const int64_t out_off = a.out_blk_off[q];
@@ -622,29 +624,29 @@ __device__ __forceinline__ void oz_pass(const NumericArgs &a, int64_t q, int lan
     }
 }
 
-template <int MAXN, bool HM, bool HKS>
+template <int MAXN, bool HM, bool HKS, bool WT>
 __device__ __forceinline__ void oz_row(const NumericArgs &a, int64_t q, int lane, int mt0, int NT, int pn, uint32_t *ring) {
     for (int nt0 = 0; nt0 < NT; nt0 += pn) {
         const int left = min(NT - nt0, pn);
-        if (MAXN == 1 || left == 1) oz_pass<1, MAXN, HM, HKS>(a, q, lane, mt0, nt0, ring);
+        if (MAXN == 1 || left == 1) oz_pass<1, MAXN, HM, HKS, WT>(a, q, lane, mt0, nt0, ring);
         else if constexpr (MAXN >= 2) {
-            if (MAXN == 2 || left == 2) oz_pass<2, MAXN, HM, HKS>(a, q, lane, mt0, nt0, ring);
-            else if constexpr (MAXN >= 3) oz_pass<3, MAXN, HM, HKS>(a, q, lane, mt0, nt0, ring);
+            if (MAXN == 2 || left == 2) oz_pass<2, MAXN, HM, HKS, WT>(a, q, lane, mt0, nt0, ring);
+            else if constexpr (MAXN >= 3) oz_pass<3, MAXN, HM, HKS, WT>(a, q, lane, mt0, nt0, ring);
         }
     }
 }
 
-// the half tile row of a block (HM) or its whole ones
-template <int MAXN, bool HM, bool HKS>
+// the half tile row of a block (HM) or its whole ones; all as whole ones (WT)
+template <int MAXN, bool HM, bool HKS, bool WT>
 __device__ __forceinline__ void oz_item(const NumericArgs &a, int64_t q, int lane, uint32_t *ring) {
     const int32_t orc = a.out_blk_rc[q];
     const int R = rc_rows(orc), NT = (rc_cols(orc) + 7) >> 3;
     const int pn = MAXN == 3 ? 3 : MAXN == 1 ? 1 : (a.pass_nt == 1 ? 1 : 2);
-    const int whole = (R + 7) >> 4;
+    const int whole = WT ? (R + 15) >> 4 : (R + 7) >> 4;
     if constexpr (HM) {
-        if (half_rows(R)) oz_row<MAXN, true, HKS>(a, q, lane, whole, NT, pn, ring);
+        if (half_rows(R)) oz_row<MAXN, true, HKS, WT>(a, q, lane, whole, NT, pn, ring);
     } else {
-        for (int mt0 = 0; mt0 < whole; ++mt0) oz_row<MAXN, false, HKS>(a, q, lane, mt0, NT, pn, ring);
+        for (int mt0 = 0; mt0 < whole; ++mt0) oz_row<MAXN, false, HKS, WT>(a, q, lane, mt0, NT, pn, ring);
     }
 }
 
@@ -653,7 +655,7 @@ __device__ __forceinline__ void oz_item(const NumericArgs &a, int64_t q, int lan
 // products (497 block rows of 23, 5 products a block: 7.1 ms, 5.2 before).
 // Items [0, n0): a warp each on the tensor cores; items [n0, n_items): tiny
 // blocks one per lane with plain FP64 FMA (exact enough, no slicing needed).
-template <int MAXN, bool HM, bool HKS>
+template <int MAXN, bool HM, bool HKS, bool WT>
 __global__ void __launch_bounds__(kThreadsNum) k_numeric_oz(NumericArgs a) {
     extern __shared__ __align__(16) uint32_t oz_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -675,7 +677,7 @@ __global__ void __launch_bounds__(kThreadsNum) k_numeric_oz(NumericArgs a) {
         int64_t q = t;
         if (a.item_order) q = (int64_t)((uint32_t)a.item_order[q] & 0x7fffffffu);
         BSM_DBG_WARP_SKIP(a, q, lane)
-        oz_item<MAXN, HM, HKS>(a, q, lane, ring);
+        oz_item<MAXN, HM, HKS, WT>(a, q, lane, ring);
     }
 }
 
@@ -738,13 +740,13 @@ __device__ __forceinline__ double elem(const T *b, int R, int Tn, int trans, int
 }
 
 // words of one block's packing
-__device__ __forceinline__ int64_t pack_words(int R, int C, int role_y, int prec) {
+__device__ __forceinline__ int64_t pack_words(int R, int C, int role_y, int prec, bool whole) {
     const int K = (prec == BSM_P_TF32x3) ? 8 : 16;
     if (prec == BSM_P_OZAKI) {
         const int T = role_y ? R : C;
-        const int hk = ((T - 1) & 15) < 8, kf = (T + 15) / 16 - hk;  // half and whole k-steps
+        const int hk = !whole && ((T - 1) & 15) < 8, kf = (T + 15) / 16 - hk;  // half and whole k-steps
         return role_y ? (int64_t)kf * oz_ystep<false>(C) + hk * oz_ystep<true>(C)
-                      : (int64_t)kf * oz_xstep<false>(R) + hk * oz_xstep<true>(R);
+                      : (int64_t)kf * (whole ? oz_xstep_whole(R) : oz_xstep<false>(R)) + hk * oz_xstep<true>(R);
     }
     if (!role_y) {
         const int XW = prec == BSM_P_BF16x6 ? 12 : 8;
@@ -761,14 +763,20 @@ __device__ __forceinline__ void logical_dims(int32_t rc, int trans, int &rows, i
     cols = trans ? rc_rows(rc) : rc_cols(rc);
 }
 
-__global__ void k_pack_sizes(int64_t nnzb, const int32_t *blk_rc, int role_y, int trans, int prec,
-                             int64_t *words) {
+__global__ void k_pack_sizes(int64_t nnzb, const int32_t *blk_rc, int role_y, int trans, int prec, bool whole,
+                             int64_t *words, unsigned long long *other) {
+    unsigned long long sum = 0;
     for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nnzb;
          b += (int64_t)gridDim.x * blockDim.x) {
         int rows, cols;
         logical_dims(blk_rc[b], trans, rows, cols);
-        words[b] = pack_words(rows, cols, role_y, prec);
+        words[b] = pack_words(rows, cols, role_y, prec, whole);
+        if (other) sum += (unsigned long long)pack_words(rows, cols, role_y, prec, !whole);
     }
+    if (!other) return;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if ((threadIdx.x & 31) == 0 && sum) atomicAdd(other, sum);
 }
 
 // one warp per block; lane L writes its fragment words of every tile
@@ -947,6 +955,7 @@ __device__ __forceinline__ void oz_slices(double x, int e, uint32_t (&out)[kOzSl
 // Ozaki fragment planes of FP64 data: the tiles of k_pack's BF16 layout with
 // kOzSlices planes, chunk-major inside a tile; X element (r, k) uses the
 // exponent of line line0[b] + r, Y element (k, n) that of line line0[b] + n.
+template <bool WHOLE>
 __global__ void k_pack_oz(int64_t nnzb, const int64_t *blk_off, const int32_t *blk_rc, const double *data,
                           int role_y, int trans, const int64_t *pack_off, uint32_t *pack, const int32_t *line0,
                           const int32_t *exps, const int32_t *status) {
@@ -966,8 +975,8 @@ __global__ void k_pack_oz(int64_t nnzb, const int64_t *blk_off, const int32_t *b
             const int MT = (rows + 15) / 16, KT = (cols + 15) / 16;
             for (int kt = 0; kt < KT; ++kt)
                 for (int mt = 0; mt < MT; ++mt) {
-                    const bool hk = cols - 16 * kt <= 8, hm = rows - 16 * mt <= 8;
-                    uint32_t *w = dst + kt * oz_xstep<false>(rows) + mt * (32 * (hk ? kOzHW : kOzXW)) + 4 * lane;
+                    const bool hk = !WHOLE && cols - 16 * kt <= 8, hm = !WHOLE && rows - 16 * mt <= 8;
+                    uint32_t *w = dst + kt * (WHOLE ? oz_xstep_whole(rows) : oz_xstep<false>(rows)) + mt * (32 * (hk ? kOzHW : kOzXW)) + 4 * lane;
                     const int r0 = mt * 16 + g, k0 = kt * 16;
                     const int rr[4] = {r0, r0 + 8, r0, r0 + 8};
                     const int kk[4] = {k0 + 2 * t4, k0 + 2 * t4, k0 + 2 * t4 + 8, k0 + 2 * t4 + 8};
@@ -991,7 +1000,7 @@ __global__ void k_pack_oz(int64_t nnzb, const int64_t *blk_off, const int32_t *b
             const int KT = (rows + 15) / 16, NT = (cols + 7) / 8;
             for (int kt = 0; kt < KT; ++kt)
                 for (int nt = 0; nt < NT; ++nt) {
-                    const bool hk = rows - 16 * kt <= 8;
+                    const bool hk = !WHOLE && rows - 16 * kt <= 8;
                     uint32_t *w = dst + kt * oz_ystep<false>(cols) + nt * (32 * (hk ? kOzQW : kOzYW)) + 4 * lane;
                     const int n0 = nt * 8 + g, k0 = kt * 16;
                     const int e = n0 < cols ? exps[l0 + n0] - 1023 : 0;
@@ -1059,14 +1068,14 @@ __global__ void k_mark_variant(int64_t n, int32_t *order, const int32_t *blk_rc,
     if (marked && cnt) atomicAdd(marked, cnt);
 }
 
-template <int MAXN, bool HM, bool HKS>
+template <int MAXN, bool HM, bool HKS, bool WT = false>
 cudaError_t launch_oz_inst(const NumericArgs &a, cudaStream_t s, int threads, int *grid) {
     const size_t smem = sizeof(uint32_t) * (size_t)oz_ring_words_per_warp<MAXN>() * (threads / 32);
     cudaError_t e =
-        cudaFuncSetAttribute(k_numeric_oz<MAXN, HM, HKS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_numeric_oz<MAXN, HM, HKS, WT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    *grid = persistent_grid(k_numeric_oz<MAXN, HM, HKS>, a.n_items, smem, threads, a.ctas_per_sm);
-    k_numeric_oz<MAXN, HM, HKS><<<*grid, threads, smem, s>>>(a);
+    *grid = persistent_grid(k_numeric_oz<MAXN, HM, HKS, WT>, a.n_items, smem, threads, a.ctas_per_sm);
+    k_numeric_oz<MAXN, HM, HKS, WT><<<*grid, threads, smem, s>>>(a);
     count_launch(1);
     return cudaGetLastError();
 }
@@ -1082,6 +1091,7 @@ cudaError_t launch_oz_rows(const NumericArgs &a, cudaStream_t s, int threads, in
 
 template <int MAXN>
 cudaError_t launch_oz(const NumericArgs &a, cudaStream_t s, int threads, int *grid) {
+    if (a.half_mask & kAllWhole) return launch_oz_inst<MAXN, false, false, true>(a, s, threads, grid);
     cudaError_t e = cudaSuccess;
     if (a.half_mask & kHalfRows) e = launch_oz_rows<MAXN, true>(a, s, threads, grid);
     if (e == cudaSuccess && (a.half_mask & kWholeRows)) e = launch_oz_rows<MAXN, false>(a, s, threads, grid);
@@ -1249,17 +1259,17 @@ cudaError_t launch_mark_variant(int64_t n, int32_t *order, const int32_t *blk_rc
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_sizes(const bsm_mat *M, int role_y, int trans, int prec, int64_t *pack_words,
-                              cudaStream_t s) {
+cudaError_t launch_pack_sizes(const bsm_mat *M, int role_y, int trans, int prec, bool whole, int64_t *pack_words,
+                              unsigned long long *other, cudaStream_t s) {
     if (M->nnzb == 0) return cudaSuccess;
     int64_t g = (M->nnzb + 255) / 256;
     if (g > 152 * 32) g = 152 * 32;
-    k_pack_sizes<<<(unsigned)g, 256, 0, s>>>(M->nnzb, M->blk_rc, role_y, trans, prec, pack_words);
+    k_pack_sizes<<<(unsigned)g, 256, 0, s>>>(M->nnzb, M->blk_rc, role_y, trans, prec, whole, pack_words, other);
     count_launch(1);
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack(const bsm_mat *M, int role_y, int trans, int prec, const int64_t *pack_off,
+cudaError_t launch_pack(const bsm_mat *M, int role_y, int trans, int prec, bool whole, const int64_t *pack_off,
                         void *pack, const int32_t *status, cudaStream_t s, const int32_t *line0,
                         const int32_t *exps) {
     if (M->nnzb == 0) return cudaSuccess;
@@ -1269,8 +1279,13 @@ cudaError_t launch_pack(const bsm_mat *M, int role_y, int trans, int prec, const
     const bool f64 = M->dtype == BSM_FP64;
     if (prec == BSM_P_OZAKI) {
         if (!f64 || !line0 || !exps) return cudaErrorInvalidValue;
-        k_pack_oz<<<(unsigned)g, 256, 0, s>>>(M->nnzb, M->blk_off, M->blk_rc, static_cast<const double *>(M->data),
-                                              role_y, trans, pack_off, p, line0, exps, status);
+        const double *d = static_cast<const double *>(M->data);
+        if (whole)
+            k_pack_oz<true><<<(unsigned)g, 256, 0, s>>>(M->nnzb, M->blk_off, M->blk_rc, d, role_y, trans, pack_off, p,
+                                                        line0, exps, status);
+        else
+            k_pack_oz<false><<<(unsigned)g, 256, 0, s>>>(M->nnzb, M->blk_off, M->blk_rc, d, role_y, trans, pack_off, p,
+                                                         line0, exps, status);
         count_launch(1);
         return cudaGetLastError();
     }

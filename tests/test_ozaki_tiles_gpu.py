@@ -51,3 +51,39 @@ def test_sizes(bsm, oracle, heights, inner):
                 np.testing.assert_array_equal(got, want)
             else:
                 assert rel_fro(got, want) <= 1e-13
+
+
+@pytest.mark.parametrize("nb,occ", [(60, 0.08), (60, 0.5), (150, 0.3), (250, 0.13)],
+                         ids=["whole", "half", "half_many", "whole_many"])
+@pytest.mark.parametrize("heights", [(23,), (5, 13, 23), (17, 40, 6)], ids=str)
+@pytest.mark.parametrize("band", [False, True], ids=["uniform", "band"])
+def test_whole_and_half_layouts(bsm, oracle, band, heights, nb, occ):
+    """Below five products a block the operands are packed in whole tiles, else in half ones where they end in half a
+    tile; a band has more products a block than the uniform pattern that the first guess assumes.  Small integers:
+    exact either way, forward, adjoints and a no-sync call with other values."""
+    import torch
+    rows = I.mixed_sizes(nb, heights, [1 / len(heights)] * len(heights), seed=3)
+    mid = I.mixed_sizes(nb, (5, 16, 24), [1 / 3] * 3, seed=4)
+    rng = np.random.default_rng(8)
+    if band:                       # the same number of blocks, in a band twice as wide as full
+        near = [(i, j) for i in range(nb) for j in range(nb) if abs(i - j) <= nb * occ]
+        Ah, Bh = (I.assemble(x, y, *np.array([p for p in near if rng.random() < 0.5]).T, None, seed=s)
+                  for x, y, s in ((rows, mid, 6), (mid, rows, 7)))
+    else:
+        Ah, Bh = random_bcsr(rows, mid, occ, seed=6), random_bcsr(mid, rows, occ, seed=7)
+    for X in (Ah, Bh):
+        X.data[:] = rng.integers(-8, 9, len(X.data))
+    A, B = bsm.Matrix.from_host(Ah), bsm.Matrix.from_host(Bh)
+    C = bsm.multiply(1.0, A, B, prec="ozaki")
+    ref = oracle.multiply(1.0, Ah, Bh)
+    np.testing.assert_array_equal(C.pattern()[1], ref.C.col_idx)
+    np.testing.assert_array_equal(C.data_host(), ref.C.data)
+    G = rng.integers(-8, 9, ref.C.data_len).astype(np.float64)
+    dA, dB = (torch.full((len(X.data),), np.nan, dtype=torch.float64, device="cuda") for X in (Ah, Bh))
+    bsm.multiply_backward(1.0, C, torch.tensor(G, device="cuda"), A, B, dA, dB, prec="ozaki")
+    for got, want in zip((dA, dB), oracle.multiply_backward(1.0, Ah, Bh, ref.C, G, ref.prods)):
+        np.testing.assert_array_equal(got.cpu().numpy(), want)
+    Ah.data[:] = rng.integers(-8, 9, len(Ah.data))
+    A.set_data(Ah.data)
+    bsm.multiply(1.0, A, B, Cm=C, prec="ozaki", no_sync=True)
+    np.testing.assert_array_equal(C.data_host(), oracle.multiply(1.0, Ah, Bh).C.data)
