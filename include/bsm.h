@@ -247,9 +247,9 @@ bsm_status bsm_get_variant(int32_t prec, int32_t m, int32_t n, int32_t *variant)
  *                        default: a kernel instance per height class of the
  *                        output blocks, over 24 rows, 17 to 24, 9 to 16 and at
  *                        most 8 -- fewer registers, more warps per SM -- one
- *                        launch each; 1 or 2 runs every block in one instance
- *                        for any height), FP64_DMMA 1..3 (default 3, 8-row
- *                        tiles)
+ *                        launch each, or one for all where the blocks are few;
+ *                        1 or 2 runs every block in one instance for any
+ *                        height), FP64_DMMA 1..3 (default 3, 8-row tiles)
  *   BSM_TUNE_PASS_NT     along the columns: split paths 1..3 (default 3,
  *                        8-column tiles), OZAKI 1..3 (default 3; 1 and 2 run
  *                        a kernel instance with a smaller staging ring and

@@ -13,7 +13,8 @@
 //
 // Two arithmetic paths:
 //   * CUDA cores: FP64 FMA; one lane owns a fixed set of output elements (the
-//     plain FP64 path is in k_group.cu, FP32 data in k_tile.cu).
+//     plain FP64 path is in k_group.cu, FP32 data in k_tile.cu, few blocks
+//     of either in k_warp.cu).
 //   * Tensor cores (mma.sync m16n8k8 TF32 / m16n8k16 BF16): operands were
 //     split beforehand into 2 or 3 narrow pieces (hi, lo[, lo2]) and packed
 //     in mma fragment order; the cross products of the pieces accumulate in
